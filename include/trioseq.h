@@ -123,7 +123,9 @@ trioseq_status trioseq_plan(const trioseq_scoring* scoring, uint32_t max_len_hin
  * Arguments: scoring as for trioseq_plan; gap_open <= 0 (>= -2^20); flags must be
  * TRIOSEQ_GLOBAL. The plan serves trioseq_align_batch and the device-resident batch calls in
  * score-only mode (traceback: ENOTIMPL); trioseq_plan_autotune has nothing to choose. The
- * kernel keeps 13 int32 states per cell and sweeps anti-diagonal planes (one CTA per triplet).
+ * kernel keeps 13 values per cell in the linear engine's column tasks, two triplets per register
+ * when a batch's values fit 16 bits; a triplet whose boundary records (2.5 bytes per cell of the
+ * cube, 1.25 packed) exceed the plan's budget (trioseq_batch_slabs) sweeps anti-diagonal planes.
  * Errors: EINVAL (as trioseq_plan, gap_open out of range, other flags), ENOMEM, ECUDA;
  * EOVERFLOW at batch time when (3 max|sub| + 3|gap| + 3|gap_open|) * (a+b+c) >= 2^29. */
 trioseq_status trioseq_plan_affine(const trioseq_scoring* scoring, int32_t gap_open,

@@ -145,7 +145,33 @@ struct WalkParams {
 
 // Affine gaps (affine.cu): natural gap costs, 13 reachable states per cell, score only.
 constexpr int kAffineStates = 13;
+// Column tasks of affine_kernel (4 x 4 cells per lane) and its boundary records: per slice, each
+// lane column's corner values and 6 values per cell of the last row (j-record), 6 values per cell
+// of the last column (k-record).
+constexpr int kAffineWJ = kPR * 4, kAffineWK = kPC * 4;
+constexpr int kAffineRecJ = kPC * (4 + 6 * 4), kAffineRecK = kPR * 6 * 4;
 struct AffineParams {
+  const TripDesc* desc;
+  const Task* tasks;      // column tasks of this launch, producers first
+  int32_t ntasks;
+  int32_t KP;
+  const int8_t* seq;
+  const int32_t* sig;     // KP x KP table of sigma''
+  int32_t* faces;
+  int32_t* progress;      // one published step count per task, zeroed before launch
+  int32_t* queue;         // zeroed before launch
+  int32_t* scores;
+  int32_t* err;
+  int32_t TI;
+  int64_t wait_ns;
+  int32_t go1, go2;       // gamma and 2 gamma (packed: in both halves)
+  int32_t neg;            // -infinity (packed: 4 |gamma| in both halves)
+  int32_t one;            // 1, as a launch argument
+};
+size_t affine_smem_bytes(int KP, bool pk);
+int affine_occupancy(bool pk, size_t smem, int* blocks_per_sm);
+int launch_affine(bool pk, const AffineParams& p, int grid, size_t smem, void* stream);
+struct AffinePlaneParams {
   const TripDesc* desc;
   const Task* tasks;      // queue: one entry per triplet (Task.trip), largest cube first
   int32_t n;
@@ -158,8 +184,8 @@ struct AffineParams {
   int32_t* queue;         // zeroed before launch
   int32_t* scores;
 };
-int affine_occupancy(int* blocks_per_sm);
-int launch_affine(const AffineParams& p, int grid, void* stream);
+int affine_plane_occupancy(int* blocks_per_sm);
+int launch_affine_plane(const AffinePlaneParams& p, int grid, void* stream);
 
 // Host-side launchers implemented in kernels.cu. `at` is the alignment type (kGlobal, ...);
 // semi-global and local exist for score mode (tb = false) only, and their scores are

@@ -271,7 +271,10 @@ struct trioseq_batch_s {
   size_t smem = 0;
   int TI = 8;  // progress-publication interval of this batch's launches
   int packed = 0;  // packed int16x2 mode (0: none, 1: signed, 2: biased): two triplets per task
-  int64_t affine_cells = 0;  // affine model: cells of the largest (j, k) plane
+  // affine model: the launches of a run as (first task, number of tasks); none when it runs over
+  // planes, whose largest has affine_cells cells
+  std::vector<std::pair<size_t, size_t>> affine_chunks;
+  int64_t affine_cells = 0;
   // Slab mode (one triplet whose records, or codes, would not fit at once): the cube runs as
   // nslab launches of `slab` slices, chained through planes of plane_ints int32 each.
   int slab = 0, nslab = 0;
@@ -344,10 +347,10 @@ void layout_inputs(trioseq_batch_s* bt) {
   bt->inputs_bytes = off;
 }
 
-// Affine-gap batch (affine.cu): one queue entry per triplet, largest cube first; each CTA of
-// the persistent launch sweeps its triplets' anti-diagonal planes in four rotating plane
-// buffers of 13 int32 states per cell. Score only.
-trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt) {
+// Affine-gap batch over anti-diagonal planes (affine_plane_kernel): one queue entry per triplet,
+// largest cube first; each CTA of the persistent launch sweeps its triplets' planes in four
+// rotating plane buffers of 13 int32 states per cell.
+trioseq_status build_affine_planes(trioseq_plan_s* plan, trioseq_batch_s* bt) {
   const size_t n = bt->n;
   std::vector<int32_t> order(n);
   int64_t maxcells = 1;
@@ -364,11 +367,123 @@ trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt) {
   bt->tasks.clear();
   for (const int32_t t : order) bt->tasks.push_back(Task{t, 0, 0, 0});
   int bpm = 0;
-  if (affine_occupancy(&bpm) != 0 || bpm <= 0) return TRIOSEQ_ECUDA;
+  if (affine_plane_occupancy(&bpm) != 0 || bpm <= 0) return TRIOSEQ_ECUDA;
   bt->grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)plan->sms * bpm, n));
   bt->affine_cells = maxcells;
   bt->face_ints = (size_t)bt->grid * 4 * (size_t)maxcells * 16;  // 16 int32 per cell (13 used)
+  layout_inputs(bt);
+  return TRIOSEQ_OK;
+}
+
+// Affine-gap batch (affine.cu). Units of one triplet, or two per register when every pair fits
+// the 16-bit halves; column tasks in the order of the linear engine (anti-diagonal, then largest
+// cube first). The boundary records take 2.5 bytes per cell of the grid, so large batches run as
+// chunks, one launch after another over the same records: 4 GB hold about ten waves of tasks of
+// 200-residue triplets, so the tail of a chunk costs little. A triplet whose records exceed the
+// plan's budget runs over planes instead (64 bytes per cell of a (j, k) plane).
+trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt) {
+  const size_t n = bt->n;
   bt->seq_bytes = bt->seq.size();
+  bt->affine_chunks.clear();
+  bt->affine_cells = 0;
+  const auto volume = [&](int32_t t) {
+    const TripDesc& d = bt->desc[t];
+    return (double)(d.len[0] + 1) * (d.len[1] + 1) * (d.len[2] + 1);
+  };
+  std::vector<int32_t> order(n);
+  for (size_t t = 0; t < n; t++) order[t] = (int32_t)t;
+  std::vector<std::pair<int32_t, int32_t>> units;
+  // Packed: sigma'' >= 0, every value of the pair's grid below 2^15 (engine.h), and -infinity
+  // (4 |gamma|, plus at most three sigma'') below the smallest real value 2^14 - 8 |gamma|.
+  const int32_t go = -plan->gap_open;
+  if (n >= 2 && plan->packed16 && plan->sig2_nonneg &&
+      12 * (int64_t)go + 3 * plan->max_abs_sig2 < (1 << 14)) {
+    const auto cls = [&](int32_t t) {
+      const TripDesc& d = bt->desc[t];
+      return std::make_tuple((d.len[1] + kAffineWJ) / kAffineWJ,
+                             (d.len[2] + kAffineWK) / kAffineWK, d.len[0]);
+    };
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int32_t x, int32_t y) { return cls(x) < cls(y); });
+    bool fits = true;
+    for (size_t u = 0; u < n && fits; u += 2) {
+      const int32_t t0 = order[u], t1 = u + 1 < n ? order[u + 1] : order[u];
+      int64_t gsum = 0;
+      for (int q = 0; q < 3; q++)
+        gsum += std::max(bt->desc[t0].len[q], bt->desc[t1].len[q]);
+      fits = (int64_t)plan->max_abs_sig2 * (gsum + 3) < (1 << 14);
+      units.emplace_back(t0, t1);
+    }
+    if (!fits) units.clear();
+  }
+  bt->packed = units.empty() ? 0 : 2;
+  if (units.empty())
+    for (size_t t = 0; t < n; t++) units.emplace_back((int32_t)t, -1);
+  // grids, then chunks of units (largest first) whose records share one buffer
+  for (const auto& un : units) {
+    TripDesc& d = bt->desc[un.first];
+    if (un.second >= 0) {
+      const TripDesc& h = bt->desc[un.second];
+      for (int q = 0; q < 3; q++) d.glen[q] = std::max(d.len[q], h.len[q]);
+      d.pair = un.second;
+    }
+    d.nJ = (d.glen[1] + kAffineWJ) / kAffineWJ;
+    d.nK = (d.glen[2] + kAffineWK) / kAffineWK;
+    d.T = d.glen[0] + 1 + (kPR - 1) + (kPC - 1);
+  }
+  std::stable_sort(units.begin(), units.end(), [&](const auto& x, const auto& y) {
+    return volume(x.first) > volume(y.first);
+  });
+  const auto records = [&](const TripDesc& d) {  // ints
+    return (size_t)d.nJ * d.nK * (size_t)(d.glen[0] + 1) * (size_t)(kAffineRecJ + kAffineRecK);
+  };
+  const size_t budget = plan->slab_budget / 4;
+  size_t limit = std::min(budget, (size_t)1 << 30);  // ints
+  for (const auto& un : units) {
+    const size_t rec = records(bt->desc[un.first]);
+    if (rec > budget) {
+      for (size_t t = 0; t < n; t++) {
+        for (int q = 0; q < 3; q++) bt->desc[t].glen[q] = bt->desc[t].len[q];
+        bt->desc[t].pair = -1;
+      }
+      bt->packed = 0;
+      return build_affine_planes(plan, bt);
+    }
+    limit = std::max(limit, rec);
+  }
+  bt->tasks.clear();
+  bt->face_ints = 4;
+  int64_t prog = 0;
+  for (size_t u0 = 0; u0 < units.size();) {
+    size_t face = 0, u1 = u0;
+    int maxD = 0;
+    for (; u1 < units.size(); u1++) {
+      TripDesc& d = bt->desc[units[u1].first];
+      const size_t ntask = (size_t)d.nJ * d.nK, A = (size_t)d.glen[0] + 1;
+      if (u1 > u0 && face + records(d) > limit) break;
+      d.oj_off = (int64_t)face;
+      d.ok_off = (int64_t)(face + ntask * A * kAffineRecJ);
+      face += records(d);
+      d.prog_base = prog;
+      prog += (int64_t)ntask;
+      maxD = std::max(maxD, d.nJ + d.nK - 2);
+    }
+    bt->face_ints = std::max(bt->face_ints, face);
+    const size_t first = bt->tasks.size();
+    for (int D = 0; D <= maxD; D++)
+      for (size_t u = u0; u < u1; u++) {
+        const int32_t t = units[u].first;
+        const TripDesc& d = bt->desc[t];
+        for (int J = std::max(0, D - d.nK + 1); J <= std::min(D, d.nJ - 1); J++)
+          bt->tasks.push_back(Task{t, J, D - J, 0});
+      }
+    bt->affine_chunks.emplace_back(first, bt->tasks.size() - first);
+    u0 = u1;
+  }
+  bt->smem = affine_smem_bytes(plan->KP, bt->packed != 0);
+  int bpm = 0;
+  if (affine_occupancy(bt->packed != 0, bt->smem, &bpm) != 0 || bpm <= 0) return TRIOSEQ_ECUDA;
+  bt->grid = plan->sms * bpm;
   layout_inputs(bt);
   return TRIOSEQ_OK;
 }
@@ -794,22 +909,53 @@ trioseq_status run(trioseq_batch_s* bt, cudaStream_t st) {
   if (e != cudaSuccess) return cuda_status(e);
   if (bt->n == 0) return TRIOSEQ_OK;
   char* in = ws.inputs.as<char>();
-  if (plan->affine) {  // affine gaps (affine.cu): score only, one CTA per triplet at a time
-    AffineParams ap{};
-    ap.desc = reinterpret_cast<const TripDesc*>(in + bt->off_desc);
-    ap.tasks = reinterpret_cast<const Task*>(in + bt->off_tasks);
-    ap.n = (int32_t)bt->tasks.size();
-    ap.KP = plan->KP;
-    ap.seq = reinterpret_cast<const int8_t*>(in);
-    ap.sub = plan->sig_affine.as<int32_t>();
-    ap.gap = plan->gap;
-    ap.gap_open = plan->gap_open;
-    ap.planes = ws.faces.as<int32_t>();
-    ap.plane_cells = bt->affine_cells;
-    ap.queue = queue;
-    ap.scores = ws.scores.as<int32_t>();
+  if (plan->affine) {  // affine gaps (affine.cu): score only
+    const TripDesc* desc = reinterpret_cast<const TripDesc*>(in + bt->off_desc);
+    const Task* tasks = reinterpret_cast<const Task*>(in + bt->off_tasks);
     if (bt->profile && record(bt->ev[0], st) != cudaSuccess) return cuda_status(cudaGetLastError());
-    if (launch_affine(ap, bt->grid, st) != 0) return cuda_status(cudaGetLastError());
+    if (bt->affine_cells) {
+      AffinePlaneParams ap{};
+      ap.desc = desc;
+      ap.tasks = tasks;
+      ap.n = (int32_t)bt->tasks.size();
+      ap.KP = plan->KP;
+      ap.seq = reinterpret_cast<const int8_t*>(in);
+      ap.sub = plan->sig_affine.as<int32_t>();
+      ap.gap = plan->gap;
+      ap.gap_open = plan->gap_open;
+      ap.planes = ws.faces.as<int32_t>();
+      ap.plane_cells = bt->affine_cells;
+      ap.queue = queue;
+      ap.scores = ws.scores.as<int32_t>();
+      if (launch_affine_plane(ap, bt->grid, st) != 0) return cuda_status(cudaGetLastError());
+    }
+    for (size_t ch = 0; ch < bt->affine_chunks.size(); ch++) {
+      const auto& [first, count] = bt->affine_chunks[ch];
+      if (ch && (e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st)) != cudaSuccess)
+        return cuda_status(e);
+      const bool pk = bt->packed != 0;
+      const auto both = [&](int32_t v) { return pk ? (v & 0xffff) | (int32_t)((uint32_t)v << 16) : v; };
+      AffineParams ap{};
+      ap.desc = desc;
+      ap.tasks = tasks + first;
+      ap.ntasks = (int32_t)count;
+      ap.KP = plan->KP;
+      ap.seq = reinterpret_cast<const int8_t*>(in);
+      ap.sig = plan->sig_score.as<int32_t>();
+      ap.faces = ws.faces.as<int32_t>();
+      ap.progress = prog;
+      ap.queue = queue;
+      ap.scores = ws.scores.as<int32_t>();
+      ap.err = err;
+      ap.TI = std::max(1, bt->TI);
+      ap.wait_ns = plan->wait_ns;
+      ap.go1 = both(plan->gap_open);
+      ap.go2 = both(2 * plan->gap_open);
+      ap.neg = pk ? both(-4 * plan->gap_open) : kNeg;
+      ap.one = 1;
+      if (launch_affine(pk, ap, bt->grid, bt->smem, st) != 0)
+        return cuda_status(cudaGetLastError());
+    }
     if (bt->profile) {
       if (record(bt->ev[1], st) != cudaSuccess || record(bt->ev[2], st) != cudaSuccess)
         return cuda_status(cudaGetLastError());
@@ -1380,7 +1526,8 @@ trioseq_status trioseq_batch_kernel(trioseq_batch_t bt, char* name, size_t cap) 
     const int nj = bt->var.nj, nk = bt->var.nk;
     char buf[160];
     if (bt->plan->affine)
-      std::snprintf(buf, sizeof buf, "affine_kernel tile plane");
+      std::snprintf(buf, sizeof buf, bt->affine_cells ? "affine_plane_kernel tile plane"
+                                                        : "affine_kernel tile 4x4");
     else if (bt->packed >= 3)
       std::snprintf(buf, sizeof buf, "wavefront_vl_kernel<%d,%d,%d> tile %dx%d%s", nj, nk / 2,
                     bt->packed - 3, nj, nk,
