@@ -102,12 +102,13 @@ typedef struct trioseq_plan_s* trioseq_plan_t;
  * TRIOSEQ_LOCAL; every call on the plan (batches, autotuner, server) uses that type.
  * Tuning read from the environment when the plan is created (none changes a result):
  * TRIOSEQ_SCORE_TILE forces the score tile ("8x8", "4x8", "4x4", or the two-cells-per-register
- * "8x16", "8x8v", "8x16s", "8x16t"; work those cannot take runs on the int32 8x8 kernel) and
- * TRIOSEQ_TB_TILE the traceback tile ("8x8", "4x8", "4x4", "8x4"); TRIOSEQ_TI the progress
+ * "8x16", "8x8v", "4x8v", "8x16s", "8x16t"; work those cannot take runs on the int32 8x8 kernel) and
+ * TRIOSEQ_TB_TILE the traceback tile ("8x8", "4x8", "4x4", "8x4", or two cells per register "8x8v",
+ * "4x8v"); TRIOSEQ_TI the progress
  * interval (steps between published progress counts, default 8); TRIOSEQ_DATA_FLAGS=1/0 forces
- * the boundary records to act as their own readiness flags in traceback launches, or not (by
- * default they do for one-triplet traceback batches); TRIOSEQ_PACKED=0 disables two triplets per
- * register; TRIOSEQ_GRAPHS=0 graph replay; TRIOSEQ_PACE=0 first-wave pacing; TRIOSEQ_WAIT_MS the
+ * the boundary records to act as their own readiness flags in int32 traceback launches, or not (by
+ * default they do for one-triplet traceback batches); TRIOSEQ_PACKED=0 disables two values per
+ * register unless a tile asks for them; TRIOSEQ_GRAPHS=0 graph replay; TRIOSEQ_PACE=0 first-wave pacing; TRIOSEQ_WAIT_MS the
  * bounded waits' limit (default 2000). TRIOSEQ_CTAS_PER_SM (read per batch) caps the resident
  * CTAs per SM.
  * Errors: EINVAL (null, bad alphabet, asymmetric sub, gap > 0, unknown flags), ECUDA. */
@@ -212,8 +213,9 @@ trioseq_status trioseq_batch_info(trioseq_batch_t batch, size_t* n, uint64_t* ce
 /* trioseq_batch_packing — *per_word = how many DP cells share each register of the batch's
  * kernel: 2 in the packed int16x2 modes, else 1. Two packed modes are the integer counterpart
  * of the paper's FP16x2 arithmetic (Sec. IV-B): two triplets per register, or two column halves
- * of one triplet per register (a one-triplet batch whose score tile is 8x16 or "8x8v", see
- * trioseq_plan_autotune). A score-only global batch of two or more triplets
+ * of one triplet per register (the tiles "8x8v", "4x8v" and 8x16: the default for every batch but
+ * small ones, see trioseq_plan_autotune, when every sigma'' is >= 0 and at most 33, 30 with
+ * traceback, which is of the global type only). A score-only global batch of two or more triplets
  * is packed when every pair fits: the batch pairs triplets of the same column-task grid class,
  * and each pair's grid needs max|sigma''| * (a+b+c+3) < 2^14 on its maximal lengths. Otherwise,
  * or with TRIOSEQ_PACKED=0 set before trioseq_plan, every triplet gets its own int32 tasks.
@@ -256,14 +258,17 @@ trioseq_status trioseq_batch_timing(trioseq_batch_t batch, float ms[2]);
 /* trioseq_plan_autotune — pick the kernel variant for a class of work by measuring it.
  * Runs the sample batch (host strings, n >= 1, mode as for trioseq_align_batch) once per
  * candidate — every instantiated register tile per lane (8x8, 4x8, 4x4 cells, i.e. column blocks
- * of 32x64, 16x64 and 16x32 cells per warp, and in traceback mode also 8x4, 32x32 cells; in
- * score-only global mode with every sigma'' in [0, 33] also the two-cells-per-register tiles
- * 8x16 and 8x8v, 32x128 and 32x64 cells per warp) times
+ * of 32x64, 16x64 and 16x32 cells per warp, and in traceback mode also 8x4, 32x32 cells; with
+ * every sigma'' in [0, 33] also the two-cells-per-register tiles
+ * 8x8v, 4x8v and, score only, 8x16, 32x64, 16x64 and 32x128 cells per warp) times, for int32,
  * progress intervals of 4, 8, 16 and 32 steps —
  * times two passes of each with CUDA events on the legacy default stream, and remembers the
  * fastest in the plan for batches of the same mode, the same single-or-batch kind, and the same
  * bit length of the longest sequence. Later batches of that class use it; other classes keep
- * the defaults (8x8 score-only, 4x8 traceback, interval 8). Outputs (any may be null) report
+ * the defaults: where the scheme admits two cells per register, tile 4x8v for batches of at most
+ * two 16x64 column tasks per SM and 8x8v beyond; int32 (8x8 score-only, 4x8 traceback, interval 8)
+ * elsewhere, for batches of at most 8 such tasks, and for score batches of two triplets that do
+ * not pack. Outputs (any may be null) report
  * the choice. The plan's device memory is untouched; a temporary workspace is used.
  * Errors: EINVAL, EOVERFLOW, ENOMEM, ETIMEOUT, ECUDA. */
 trioseq_status trioseq_plan_autotune(trioseq_plan_t plan, const trioseq_triplet* sample, size_t n,

@@ -22,6 +22,9 @@ constexpr int kNeg = -(1 << 30);   // -infinity sentinel (never accumulates: see
 // A boundary-record slot not yet written (the byte 0x80 repeated): below -infinity and below any
 // key, so no stored value can equal it.
 constexpr int kRecordSentinel = (int)0x80808080u;
+// The same for the two-cells-per-register kernel, whose record words are packed halves below 0xffff
+// or bases that are multiples of 8.
+constexpr int kVlSentinel = -1;
 constexpr int kPR = 4;             // lanes of a warp along j
 constexpr int kPC = 8;             // lanes of a warp along k
 constexpr int kMaxAlphabet = 32;
@@ -52,6 +55,10 @@ constexpr int kBias16x2 = 0x40004000;
 // Cell (p, q) of the lane tile is e = p*NK + q; it lives in word e/8 at bit
 //   8*(e & 3) + 4*((e >> 2) & 1)   (the 3-bit rank in the low bits of that nibble).
 __host__ __device__ inline int code_bit(int e) { return 8 * (e & 3) + 4 * ((e >> 2) & 1); }
+// The two-cells-per-register traceback kernel (wavefront_vl.cuh) writes the same records for 4 x 16
+// virtual lanes of NJ x 4 cells, with another order inside a word: two rows of four cells, the
+// first cell of a row in its highest nibble.
+__host__ __device__ inline int vl_code_bit(int e) { return 16 * ((e >> 2) & 1) + 12 - 4 * (e & 3); }
 
 // Face records. Column task (J, K) publishes, per slice s (0..a):
 //   its last j-row in the j-record  Oj[s][0 .. WK+3]: slot 3 = M'[s][J*WJ+WJ-1][K*WK-1] (the
@@ -59,6 +66,11 @@ __host__ __device__ inline int code_bit(int e) { return 8 * (e & 3) + 4 * ((e >>
 //   its last k-column in the k-record Ok[s][0 .. WJ-1] = M'[s][J*WJ + jl][K*WK+WK-1].
 // Records of one task are contiguous: Oj at oj_off + task*(a+1)*(WK+4), Ok at
 // ok_off + task*(a+1)*WJ (int32 offsets into the face workspace).
+
+// The two-cells-per-register kernel (wavefront_vl.cuh) keeps records by producer step instead:
+// T rows of vl_rec_j(NH) and kVlRecK int32 per column task.
+constexpr int vl_rec_j(int NH) { return kPC * (NH + 2); }
+constexpr int kVlRecK = kPR * 6;
 
 struct TripDesc {
   int64_t s_off[3];    // byte offsets of S0, S1, S2 in the packed residue buffer
@@ -131,6 +143,7 @@ struct WalkParams {
   int32_t* aln_len;          // written: alignment length (the alignment is the last L bytes)
   int32_t* err;              // bit 1: corrupt code met during a walk
   int32_t NJ, NK;            // tile of the wavefront variant that wrote the codes
+  int32_t vl;                // 1: codes of virtual lanes (4 x 16 lanes of NJ x NK cells)
   // Slab walks (linear-space traceback): codes hold only the slices i_lo .. of a slab launch
   // with T_slab steps per task; state (i, j, k, n per request) carries the walk across slabs.
   // i_lo = 0, T_slab = 0 and state = null walk the whole cube from (a, b, c) in one launch.
@@ -202,17 +215,20 @@ int wavefront_occupancy(int nj, int nk, bool tb, int at, int pk, bool slab, size
 const void* wavefront_variant(int nj, int nk, int at, bool tb);
 // Kernel entry of a packed int16x2 (global, score) instantiation (kernels_packed.cu), or null.
 const void* wavefront_packed(int nj, int nk, int mode);
-// two cells of one triplet per register (wavefront_vl.cuh): nj x nk = 8 x 16 or 8 x 8 cells per
-// lane; cs = 1 or 2: the lane's sigma''(y,z) tile in shared memory (8 x 16 only; 2-warp or
+// two cells of one triplet per register (wavefront_vl.cuh): nj x nk = 8 x 16, 8 x 8 or 4 x 8 cells
+// per lane; cs = 1 or 2: the lane's sigma''(y,z) tile in shared memory (8 x 16 only; 2-warp or
 // 1-warp CTAs), 0: in registers
-const void* wavefront_vl(int nj, int nk, int cs, int at);
+// tb: traceback keys (global type, NH = 4). Null where not built.
+const void* wavefront_vl(int nj, int nk, int cs, int at, bool tb);
+const void* wavefront_vl_tb(int nj, int nk);              // kernels_vl_tb.cu
+const void* wavefront_vl_types(int nj, int nk, int at);   // kernels_vl_types.cu
 size_t wavefront_vl_smem_bytes(int nj, int nk, int KP, int cs);
 int wavefront_vl_warps(int cs);
 // Kernel entry of a slab-launch instantiation (kernels_slab.cu), or null.
 const void* wavefront_slab(int nj, int nk, bool tb);
 int launch_walk(const WalkParams& p, void* stream);
 size_t wavefront_smem_bytes(int nj, int nk, int KP, bool pk);
-// threads per CTA of a launch in packed mode pk (2 warps for pk = 4, 1 for pk = 5, else
+// threads per CTA of a launch in packed mode pk (1 warp for pk = 3 and 5, 2 for pk = 4, else
 // kWarpsPerCta)
 int wavefront_block_threads(int pk);
 

@@ -36,7 +36,8 @@ __device__ __forceinline__ int win_base(int x, int l) {
 
 // The triplet's shape comes in registers (len: the three lengths; nK: column tasks along k;
 // nJR, nKC: lane rows / columns of the task grid), read once by the caller.
-template <int W>
+// PC: lane columns of a column task (kPC, or 2 * kPC for virtual lanes).
+template <int W, int PC>
 __device__ __forceinline__ void tube_load(uint32_t* win, uint8_t (*res)[kWin], int i0, int j0,
                                           int k0, int lj, int lk, const uint32_t* codes,
                                           const int (&len)[3], int nK, int nJR, int nKC,
@@ -65,10 +66,10 @@ __device__ __forceinline__ void tube_load(uint32_t* win, uint8_t (*res)[kWin], i
     const int gc = ((k0 - sx) >> lk) + rem % kTubeC - 1;
     valid[u] = e < kTubeRecs && ii >= i_lo && gr >= 0 && gc >= 0 && gr < nJR && gc < nKC;
     if (valid[u]) {
-      const int task = (gr / kPR) * nK + (gc / kPC);
-      const int lr = gr % kPR, lcc = gc % kPC;
+      const int task = (gr / kPR) * nK + (gc / PC);
+      const int lr = gr % kPR, lcc = gc % PC;
       const uint32_t* src =
-          codes + (((int64_t)task * T + (ii - i_lo + lr + lcc)) * 32 + (lr * kPC + lcc)) * W;
+          codes + (((int64_t)task * T + (ii - i_lo + lr + lcc)) * (kPR * PC) + (lr * PC + lcc)) * W;
       if (W == 2) {
         const uint2 h = __ldcg(reinterpret_cast<const uint2*>(src));
         v[u][0] = make_uint4(h.x, h.y, 0u, 0u);
@@ -98,7 +99,7 @@ __device__ __forceinline__ void tube_load(uint32_t* win, uint8_t (*res)[kWin], i
   }
 }
 
-template <int W>
+template <int W, int PC>
 __global__ void __launch_bounds__(32) walk_kernel(const WalkParams p) {
   __shared__ uint4 win4[kTubeRecs * W / 4 + 1];
   __shared__ uint8_t res[3][kWin];
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkParams p) {
   const TripDesc& d = p.desc[p.tb_trips[q]];
   const int a = d.len[0], b = d.len[1], c = d.len[2];
   const int len[3] = {a, b, c};
-  const int nK = d.nK, nJR = d.nJ * kPR, nKC = d.nK * kPC;
+  const int nK = d.nK, nJR = d.nJ * kPR, nKC = d.nK * PC;
   const int lj = __ffs(p.NJ) - 1, lk = __ffs(p.NK) - 1;  // tile sides are powers of two
   const int8_t* const S[3] = {p.seq + d.s_off[0], p.seq + d.s_off[1], p.seq + d.s_off[2]};
   const int cap = p.row_cap[q];
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkParams p) {
   int done = start(i, j, k);
   while (!done && i >= i_lo && !bad) {
     const int i0 = i, j0 = j, k0 = k;
-    tube_load<W>(win, res, i0, j0, k0, lj, lk, codes, len, nK, nJR, nKC, S, T, i_lo, lane);
+    tube_load<W, PC>(win, res, i0, j0, k0, lj, lk, codes, len, nK, nJR, nKC, S, T, i_lo, lane);
     __syncwarp();
     // residue windows: S0[x - 1] is res[0][x - iw], and likewise for S1 and S2
     const int iw = i0 - kTubeS + 1, jw = win_base(j0, lj) + 1, kw = win_base(k0, lk) + 1;
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkParams p) {
       if ((unsigned)dr >= (unsigned)kTubeR || (unsigned)dc >= (unsigned)kTubeC) return -1;
       const int e = ((cj & ((1 << lj) - 1)) << lk) + (ck & ((1 << lk) - 1));
       const uint32_t word = win[((sx * kTubeR + dr) * kTubeC + dc) * W + (e >> 3)];
-      return (word >> code_bit(e)) & 7;
+      return (word >> (PC == kPC ? code_bit(e) : vl_code_bit(e))) & 7;
     };
     for (;;) {  // warp-uniform
       // Lane m probes the cell m diagonal moves ahead; the run is the leading lanes whose cell
@@ -248,7 +249,7 @@ const void* kptr() {
 
 const void* pick(int nj, int nk, bool tb, int at, int pk, bool slab) {
   if (slab) return (pk || at != kGlobal) ? nullptr : wavefront_slab(nj, nk, tb);
-  if (pk >= 3) return tb ? nullptr : wavefront_vl(nj, nk, pk - 3, at);
+  if (pk >= 3) return wavefront_vl(nj, nk, pk - 3, at, tb);
   if (pk) return (tb || at != kGlobal) ? nullptr : wavefront_packed(nj, nk, pk);
   if (at != kGlobal) return wavefront_variant(nj, nk, at, tb);
   if (nj == 8 && nk == 8) return tb ? kptr<8, 8, true>() : kptr<8, 8, false>();
@@ -262,7 +263,9 @@ const void* pick(int nj, int nk, bool tb, int at, int pk, bool slab) {
 
 }  // namespace
 
-int wavefront_block_threads(int pk) { return 32 * (pk >= 3 ? wavefront_vl_warps(pk - 3) : kWarpsPerCta); }
+int wavefront_block_threads(int pk) {
+  return 32 * (pk >= 3 ? wavefront_vl_warps(pk - 3) : kWarpsPerCta);
+}
 
 size_t wavefront_smem_bytes(int nj, int nk, int KP, bool pk) {
   const int WJ = kPR * nj, WK = kPC * nk;
@@ -300,9 +303,12 @@ int launch_walk(const WalkParams& p, void* stream) {
   if (p.ntb <= 0) return 0;
   const int W = p.NJ * p.NK / 8;
   cudaStream_t st = (cudaStream_t)stream;
-  if (W == 2) walk_kernel<2><<<p.ntb, 32, 0, st>>>(p);
-  else if (W == 4) walk_kernel<4><<<p.ntb, 32, 0, st>>>(p);
-  else if (W == 8) walk_kernel<8><<<p.ntb, 32, 0, st>>>(p);
+  if (p.vl && W == 4) walk_kernel<4, 2 * kPC><<<p.ntb, 32, 0, st>>>(p);
+  else if (p.vl && W == 2) walk_kernel<2, 2 * kPC><<<p.ntb, 32, 0, st>>>(p);
+  else if (p.vl) return -1;
+  else if (W == 2) walk_kernel<2, kPC><<<p.ntb, 32, 0, st>>>(p);
+  else if (W == 4) walk_kernel<4, kPC><<<p.ntb, 32, 0, st>>>(p);
+  else if (W == 8) walk_kernel<8, kPC><<<p.ntb, 32, 0, st>>>(p);
   else return -1;
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }

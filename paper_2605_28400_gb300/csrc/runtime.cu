@@ -231,6 +231,7 @@ struct trioseq_plan_s {
   int slab_slices = 0;             // forced slab height (0: chosen from the budget)
   Variant score_variant{8, 8};
   Variant tb_variant{4, 8};
+  bool score_forced = false, tb_forced = false;  // set by TRIOSEQ_SCORE_TILE / TRIOSEQ_TB_TILE
   // Autotuner cache: (mode, single triplet or batch, bit length of the longest sequence) ->
   // fastest (tile, progress interval) measured by trioseq_plan_autotune.
   struct Tuned {
@@ -270,6 +271,7 @@ struct trioseq_batch_s {
   int grid = 0;
   size_t smem = 0;
   int TI = 8;  // progress-publication interval of this batch's launches
+  bool df = false;  // boundary records are their own readiness flags
   int packed = 0;  // packed int16x2 mode (0: none, 1: signed, 2: biased): two triplets per task
   // affine model: the launches of a run as (first task, number of tasks); none when it runs over
   // planes, whose largest has affine_cells cells
@@ -488,6 +490,64 @@ trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt) {
   return TRIOSEQ_OK;
 }
 
+int plan_atype(const trioseq_batch_s* bt) { return bt->plan->atype; }
+
+// Units of the packed int16x2 mode on WJ x WK column tasks: two triplets of the same grid class each
+// (the last one with itself when n is odd), or none when some pair's grid leaves the int16 margin of
+// engine.h: max|sigma''| * (a+b+c + 3) < 2^14 on the pair's maximal lengths.
+std::vector<std::pair<int32_t, int32_t>> pack_units(const trioseq_plan_s* plan,
+                                                    const trioseq_triplet* trip, size_t n, int WJ,
+                                                    int WK) {
+  std::vector<std::pair<int32_t, int32_t>> units;
+  std::vector<int32_t> order(n);
+  for (size_t t = 0; t < n; t++) order[t] = (int32_t)t;
+  const auto cls = [&](int32_t t) {
+    const uint32_t* L = trip[t].len;
+    return std::make_tuple((L[1] + WJ) / WJ, (L[2] + WK) / WK, L[0]);
+  };
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int32_t x, int32_t y) { return cls(x) < cls(y); });
+  for (size_t u = 0; u < n; u += 2) {
+    const int32_t t0 = order[u], t1 = (u + 1 < n) ? order[u + 1] : order[u];
+    int64_t gsum = 0;
+    for (int q = 0; q < 3; q++) gsum += std::max(trip[t0].len[q], trip[t1].len[q]);
+    if ((int64_t)plan->max_abs_sig2 * (gsum + 3) >= (1 << 14)) return {};
+    units.emplace_back(t0, t1);
+  }
+  return units;
+}
+
+// Whether the tile of a plan's batches is chosen by default_variant: no forced tile, and two values per
+// register not switched off.
+bool auto_tile(const trioseq_plan_s* plan, bool tb) {
+  return !plan->affine && plan->packed16 && !(tb ? plan->tb_forced : plan->score_forced);
+}
+
+// Schemes and types the two-cells-per-register kernel admits (its range argument). Traceback keys
+// (global type) take 3 bits more.
+bool vl_admits(const trioseq_plan_s* plan, bool tb) {
+  return plan->sig2_nonneg && plan->max_abs_sig2 <= (tb ? 30 : 33) &&
+         (plan->atype == kGlobal || (!tb && -2 * plan->gap <= 33));
+}
+
+// The tile of a batch when neither the environment nor the autotuner names one: two cells of a
+// triplet per register (wavefront_vl.cuh; build_batch falls back to int32 where the scheme or the
+// budget does not admit it), 16 x 64 tasks while they number at most two per SM (more warps than 32 x 64 tasks
+// give, each with a shorter step; beyond that their records cost more than they gain), else 32 x 64.
+// Measured, kernel time (16 x 64 / 32 x 64 / int32 default): score, protein, 300 residues (95 /
+// 50 tasks) 0.19 / 0.22 / 0.50 ms; 1,000 residues (1,008 / 512) 0.80 / 0.71 / 1.74 ms; traceback, DNA, 128
+// residues (16 / 8) 0.094 / 0.119 / 0.129 ms, 1,000 residues 1.01 / 0.96 / 1.47 ms, 96 triplets of
+// 200..600 3.3 / 3.2 / 6.3 ms; 1,024 semi-global triplets of 100..300 4.8 / 4.3 / 7.2 ms.
+// Kept on int32: launches of at most 8 such tasks, where the launch itself is most of the time
+// (64 residues: 50 against 63 us), and score batches of exactly two triplets that cannot pack.
+Variant default_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n, bool tb) {
+  uint64_t tasks = 0;
+  for (size_t t = 0; t < n; t++)
+    tasks += (uint64_t)((trip[t].len[1] + 16) / 16) * ((trip[t].len[2] + 64) / 64);
+  if (tasks <= 8 || (!tb && n == 2)) return tb ? plan->tb_variant : plan->score_variant;
+  return tasks <= 2 * (uint64_t)plan->sms ? Variant{4, 8, 1} : Variant{8, 8, 1};
+}
+
 // Build the host side of a batch: encode, pack, describe, order the queue.
 trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n,
                            uint32_t mode, trioseq_batch_s* bt) {
@@ -499,6 +559,7 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   bt->mode = mode;
   bt->var = tb ? plan->tb_variant : plan->score_variant;
   bt->TI = plan->TI;
+  std::vector<std::pair<int32_t, int32_t>> units;  // (low-half triplet, high-half triplet or -1)
   {
     uint32_t maxlen = 0;
     for (size_t t = 0; t < n; t++)
@@ -511,6 +572,12 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
       if (it != plan->tuned.end()) {
         bt->var = it->second.var;
         bt->TI = it->second.TI;
+      } else if (auto_tile(plan, tb) &&
+                 !(n == 1 && plan->atype == kGlobal && plan->slab_slices > 0)) {
+        // global score batches whose pairs fit run two triplets per register on the int32 tile
+        if (!tb && plan->atype == kGlobal && n >= 2 && maxlen <= (1u << 24))
+          units = pack_units(plan, trip, n, kPR * bt->var.nj, kPC * bt->var.nk);
+        if (units.empty()) bt->var = default_variant(plan, trip, n, tb);
       }
     }
   }
@@ -522,20 +589,23 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   if (bt->var.vl) {
     // (semi-global and local too: their zero axes and floor add steps of -2*alpha, which must
     // also stay <= 33)
-    bool ok_vl = !tb && plan->sig2_nonneg && plan->max_abs_sig2 <= 33 &&
-                 (plan->atype == kGlobal || -2 * plan->gap <= 33) &&
-                 wavefront_vl(bt->var.nj, bt->var.nk, bt->var.vl - 1, plan->atype) != nullptr;
+    bool ok_vl = vl_admits(plan, tb) &&
+                 wavefront_vl(bt->var.nj, bt->var.nk, bt->var.vl - 1, plan->atype, tb) != nullptr;
     if (ok_vl) {
       const int wj = kPR * bt->var.nj, wk = kPC * bt->var.nk;
-      double rec = 0;  // int32 boundary records of all triplets: (a+1) x tasks x (WK+4 + WJ)
+      double rec = 0;  // boundary records of all triplets: steps x tasks x row
       for (size_t t = 0; t < n; t++)
-        rec += (trip[t].len[0] + 1.0) * ((trip[t].len[1] + wj) / wj) *
-               ((trip[t].len[2] + wk) / wk) * (4.0 * (wk + 4 + wj));
-      ok_vl = rec <= (double)plan->slab_budget;
+        rec += (trip[t].len[0] + 19.0) * ((trip[t].len[1] + wj) / wj) *
+               ((trip[t].len[2] + wk) / wk) * (4.0 * (vl_rec_j(bt->var.nk / 2) + kVlRecK));
+      // one traceback triplet's codes count too: beyond the budget it runs in (int32) slabs
+      if (tb && n == 1)
+        rec += (trip[0].len[0] + 19.0) * ((trip[0].len[1] + wj) / wj) *
+               ((trip[0].len[2] + wk) / wk) * (wj * wk / 2.0);
+      ok_vl = rec <= (double)plan->slab_budget && !(tb && n == 1 && plan->slab_slices > 0);
     }
     if (!ok_vl) {
       if (plan->tuning) return TRIOSEQ_ECUDA;  // the autotuner skips the candidate
-      bt->var = Variant{8, 8};
+      bt->var = tb ? Variant{4, 8} : Variant{8, 8};  // the int32 defaults
     }
   }
   const int NJ = bt->var.nj, NK = bt->var.nk;
@@ -640,37 +710,14 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   }
   // 2. Units of work: one triplet, or in packed int16x2 mode two triplets of the same column-task
   //    grid class paired in one unit (the high halves run on the grid of their maximal lengths).
-  //    Packing needs every value of the pair's grid within the int16 margin of engine.h:
-  //    max|sigma''| * (a+b+c + 3) < 2^14 on the grid's lengths.
-  std::vector<std::pair<int32_t, int32_t>> units;  // (low-half triplet, high-half triplet or -1)
   bt->packed = 0;
   const bool vl = bt->var.vl != 0;  // admitted above
   if (vl) bt->packed = 2 + bt->var.vl;  // 3: registers; 4, 5: sigma'' tile in shared memory
   const int pmode = plan->sig2_nonneg ? 2 : 1;
   if (!vl && !tb && plan->atype == kGlobal && plan->packed16 && n >= 2 &&
       wavefront_packed(NJ, NK, pmode) != nullptr) {
-    std::vector<int32_t> order(n);
-    for (size_t t = 0; t < n; t++) order[t] = (int32_t)t;
-    const auto cls = [&](int32_t t) {
-      const TripDesc& d = bt->desc[t];
-      return std::make_tuple((d.len[1] + WJ) / WJ, (d.len[2] + WK) / WK, d.len[0]);
-    };
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int32_t x, int32_t y) { return cls(x) < cls(y); });
-    bool fits = true;
-    for (size_t u = 0; u < n && fits; u += 2) {
-      const int32_t t0 = order[u], t1 = (u + 1 < n) ? order[u + 1] : order[u];
-      int64_t gsum = 0;
-      for (int q = 0; q < 3; q++)
-        gsum += std::max(bt->desc[t0].len[q], bt->desc[t1].len[q]);
-      fits = (int64_t)plan->max_abs_sig2 * (gsum + 3) < (1 << 14);
-      units.emplace_back(t0, t1);
-    }
-    if (fits) {
-      bt->packed = pmode;
-    } else {
-      units.clear();
-    }
+    if (units.empty()) units = pack_units(plan, trip, n, WJ, WK);
+    if (!units.empty()) bt->packed = pmode;
   }
   if (units.empty())  // one unit per triplet (no pairs formed)
     for (size_t t = 0; t < n; t++) units.emplace_back((int32_t)t, -1);
@@ -688,10 +735,12 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
     d.T = a + 1 + (kPR - 1) + (kPC - 1) + (vl ? kPC : 0);  // vl: 2*kPC virtual lane columns
     // boundary records of every column task: (a+1) x (WK+4) j-records, (a+1) x WJ k-records
     const size_t ntask = (size_t)d.nJ * (size_t)d.nK;
+    // (vl: by producer step, T x vl_rec_j and T x kVlRecK)
     d.oj_off = (int64_t)face;
-    face += ntask * (size_t)(a + 1) * (size_t)(WK + 4);
+    face += vl ? ntask * (size_t)d.T * (size_t)vl_rec_j(NK / 2)
+               : ntask * (size_t)(a + 1) * (size_t)(WK + 4);
     d.ok_off = (int64_t)face;
-    face += ntask * (size_t)(a + 1) * (size_t)WJ;
+    face += vl ? ntask * (size_t)d.T * (size_t)kVlRecK : ntask * (size_t)(a + 1) * (size_t)WJ;
     face = align_up(face, 4);
     d.prog_base = prog;
     prog += (int64_t)d.nJ * d.nK;
@@ -818,16 +867,20 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   bt->smem = bt->packed >= 3 ? wavefront_vl_smem_bytes(NJ, NK, plan->KP, bt->packed - 3)
                              : wavefront_smem_bytes(NJ, NK, plan->KP, bt->packed != 0);
   int bpm = 0;
-  if (wavefront_occupancy(NJ, NK, tb, plan->atype, bt->packed, bt->slab > 0, bt->smem, &bpm) !=
-          0 ||
+  // Int32 traceback launches of one triplet use the records as readiness flags; TRIOSEQ_DATA_FLAGS at
+  // plan creation forces it on (1) or off (0). (The two-cells-per-register kernel always does.)
+  bt->df = tb && !vl && !bt->slab && (plan->data_flags >= 0 ? plan->data_flags != 0 : n == 1);
+  if (wavefront_occupancy(NJ, NK, tb, plan->atype, bt->packed, bt->slab > 0, bt->smem,
+                          &bpm) != 0 ||
       bpm <= 0)
     return TRIOSEQ_ECUDA;
   const int want = env_int("TRIOSEQ_CTAS_PER_SM", bpm);
   bt->grid = plan->sms * std::max(1, std::min(bpm, want));
+  if (vl)  // no CTA without a task: one that finds the queue empty still costs its start
+    bt->grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)bt->grid, bt->tasks.size()));
   return TRIOSEQ_OK;
 }
 
-int plan_atype(const trioseq_batch_s* bt) { return bt->plan->atype; }
 
 // Size the workspace and copy the inputs of `bt` into it (stream-ordered).
 // `pinned`: stage through the workspace's pinned buffer and copy asynchronously on `st` (the
@@ -980,12 +1033,11 @@ trioseq_status run(trioseq_batch_s* bt, cudaStream_t st) {
   p.wait_ns = plan->wait_ns;
   p.g2 = -2 * plan->gap;
   p.one = 1;
-  // One-triplet traceback launches, whose time is the wavefront ramp: records carry their own
+  // One-triplet int32 traceback launches, whose time is the wavefront ramp: records carry their own
   // readiness (sentinel-filled here, in the launch's stream order), so each producer-consumer
-  // level lags by its skew alone instead of also by a publication interval and a flag round
-  // trip; progress is then published only at the end of a task. TRIOSEQ_DATA_FLAGS at plan
-  // creation forces it on (1) or off (0) for every traceback launch.
-  p.data_flags = tb && !bt->slab && (plan->data_flags >= 0 ? plan->data_flags : bt->n == 1);
+  // level lags by its skew alone instead of also by a publication interval and a flag round trip;
+  // progress is then published only at the end of a task.
+  p.data_flags = bt->df;
   if (p.data_flags) {
     if ((e = cudaMemsetAsync(p.faces, 0x80, bt->face_ints * sizeof(int32_t), st)) != cudaSuccess)
       return cuda_status(e);
@@ -999,7 +1051,7 @@ trioseq_status run(trioseq_batch_s* bt, cudaStream_t st) {
     p.pace_n = bt->grid * warps_per_cta;
     p.pace_T = 1 << 20;
     p.pace_flag = prog + bt->tasks.size() + 48;
-  } else if (!bt->slab && plan->pace && !p.data_flags &&
+  } else if (!bt->slab && plan->pace && !p.data_flags && bt->packed < 3 &&
              bt->tasks.size() >= 2 * (size_t)bt->grid * warps_per_cta) {
     // pace the first wave against the progress of queue task 0, the (0,0) block of its triplet
     const TripDesc& d0 = bt->desc[bt->tasks[0].trip];
@@ -1028,7 +1080,8 @@ trioseq_status run(trioseq_batch_s* bt, cudaStream_t st) {
   w.aln_len = ws.lens.as<int32_t>();
   w.err = err;
   w.NJ = bt->var.nj;
-  w.NK = bt->var.nk;
+  w.NK = bt->var.vl ? bt->var.nk / 2 : bt->var.nk;  // virtual lanes hold half the columns
+  w.vl = bt->var.vl ? 1 : 0;
   w.atype = plan->atype;
   w.best64 = p.best64;
   w.scores = p.scores;
@@ -1081,8 +1134,8 @@ trioseq_status run(trioseq_batch_s* bt, cudaStream_t st) {
     if (bt->profile && record(bt->ev[1], st) != cudaSuccess)
       return cuda_status(cudaGetLastError());
   } else {
-    if (launch_wavefront(bt->var.nj, bt->var.nk, tb, plan->atype, bt->packed, false, p, bt->grid,
-                         bt->smem, st) != 0)
+    if (launch_wavefront(bt->var.nj, bt->var.nk, tb, plan->atype, bt->packed, false, p,
+                         bt->grid, bt->smem, st) != 0)
       return cuda_status(cudaGetLastError());
     if (bt->profile && record(bt->ev[1], st) != cudaSuccess)
       return cuda_status(cudaGetLastError());
@@ -1308,7 +1361,7 @@ trioseq_status trioseq_plan(const trioseq_scoring* sc, uint32_t max_len_hint, ui
       plan->slab_slices = std::max(0, env_int("TRIOSEQ_SLAB_SLICES", 0));
     }
     // "RxC": register tile rows x columns per lane
-    const auto parse_tile = [](const char* v, Variant* out) {
+    const auto parse_tile = [](const char* v, Variant* out, bool* forced) {
       if (!v) return;
       char* end = nullptr;
       const long rj = std::strtol(v, &end, 10);
@@ -1319,10 +1372,13 @@ trioseq_status trioseq_plan(const trioseq_scoring* sc, uint32_t max_len_hint, ui
       // 's' or 't' ("8x16s", "8x16t") its variants with the sigma''(y,z) tile in shared memory
       const char sfx = end2 ? *end2 : 0;
       const int two = sfx == 's' ? 2 : (sfx == 't' ? 3 : ((ck == 16 || sfx == 'v') ? 1 : 0));
-      if (rj > 0 && rj <= 16 && ck > 0 && ck <= 32) *out = Variant{(int)rj, (int)ck, two};
+      if (rj > 0 && rj <= 16 && ck > 0 && ck <= 32) {
+        *out = Variant{(int)rj, (int)ck, two};
+        *forced = true;
+      }
     };
-    parse_tile(std::getenv("TRIOSEQ_SCORE_TILE"), &plan->score_variant);
-    parse_tile(std::getenv("TRIOSEQ_TB_TILE"), &plan->tb_variant);
+    parse_tile(std::getenv("TRIOSEQ_SCORE_TILE"), &plan->score_variant, &plan->score_forced);
+    parse_tile(std::getenv("TRIOSEQ_TB_TILE"), &plan->tb_variant, &plan->tb_forced);
     *out = plan.release();
     return TRIOSEQ_OK;
   });
@@ -1529,8 +1585,8 @@ trioseq_status trioseq_batch_kernel(trioseq_batch_t bt, char* name, size_t cap) 
       std::snprintf(buf, sizeof buf, bt->affine_cells ? "affine_plane_kernel tile plane"
                                                         : "affine_kernel tile 4x4");
     else if (bt->packed >= 3)
-      std::snprintf(buf, sizeof buf, "wavefront_vl_kernel<%d,%d,%d> tile %dx%d%s", nj, nk / 2,
-                    bt->packed - 3, nj, nk,
+      std::snprintf(buf, sizeof buf, "wavefront_vl_kernel<%d,%d,%d%s> tile %dx%d%s", nj, nk / 2,
+                    bt->packed - 3, tb ? ",traceback" : "", nj, nk,
                     bt->packed == 4 ? "s" : (bt->packed == 5 ? "t" : (nk == 16 ? "" : "v")));
     else if (bt->packed)
       std::snprintf(buf, sizeof buf, "wavefront_kernel<%d,%d,score,global,%s> tile %dx%d", nj, nk,
@@ -1586,9 +1642,9 @@ trioseq_status trioseq_plan_autotune(trioseq_plan_t plan, const trioseq_triplet*
     }
     // candidate tiles per mode; 8x4 exists for traceback keys only
     // 8x16 and 8x8 with vl: two cells of one triplet per register
-    static const Variant kScoreTiles[] = {{8, 8},    {4, 8},    {4, 4},   {8, 16, 1},
-                                          {8, 8, 1}, {8, 16, 2}, {8, 16, 3}};
-    static const Variant kTbTiles[] = {{8, 8}, {4, 8}, {4, 4}, {8, 4}};
+    static const Variant kScoreTiles[] = {{8, 8},    {4, 8},     {4, 4},     {8, 16, 1},
+                                          {8, 8, 1}, {8, 16, 2}, {8, 16, 3}, {4, 8, 1}};
+    static const Variant kTbTiles[] = {{8, 8}, {4, 8}, {4, 4}, {8, 4}, {8, 8, 1}, {4, 8, 1}};
     static const int kTI[] = {4, 8, 16, 32};
     const bool tb_mode = mode == TRIOSEQ_WITH_TRACEBACK;
     const Variant* tiles = tb_mode ? kTbTiles : kScoreTiles;
@@ -1611,6 +1667,7 @@ trioseq_status trioseq_plan_autotune(trioseq_plan_t plan, const trioseq_triplet*
       for (size_t vi = 0; vi < ntiles; vi++) {
         const Variant& v = tiles[vi];
         for (int ti : kTI) {
+          if (v.vl && ti != kTI[0]) break;  // it publishes no progress: the interval is moot
           plan->forced = trioseq_plan_s::Tuned{v, ti};
           trioseq_batch_s bt;
           trioseq_status s = build_batch(plan, sample, n, mode, &bt);
@@ -1731,7 +1788,16 @@ size_t request_bytes(const trioseq_plan_s* plan, uint32_t mode, const uint32_t l
   const size_t a = len[0], b = len[1], c = len[2];
   const size_t nJ = (b + 1 + WJ - 1) / WJ, nK = (c + 1 + WK - 1) / WK, T = a + 1 + 10;
   size_t bytes = 4 * nJ * nK * (a + 1) * ((WK + 4) + WJ) + 4 * nJ * nK + 256 + a + b + c + 48;
-  if (tb) bytes += 4 * nJ * nK * T * 32 * W + 3 * (a + b + c) + 64;
+  if (tb) bytes += 4 * nJ * nK * T * 32 * W;
+  if (auto_tile(plan, tb) && vl_admits(plan, tb)) {  // the two-per-register tile it may run on instead
+    const size_t t16 = (b + 16) / 16 * ((c + 64) / 64), t32 = (b + 32) / 32 * ((c + 64) / 64);
+    const bool narrow = t16 <= 2 * (size_t)plan->sms;
+    const size_t vt = narrow ? t16 : t32, cells = narrow ? 16 * 64 : 32 * 64;
+    const size_t need = vt * (a + 19) * (4 * (vl_rec_j(4) + kVlRecK) + (tb ? cells / 2 : 0)) +
+                        4 * vt + 256 + a + b + c + 48;
+    bytes = std::max(bytes, need);
+  }
+  if (tb) bytes += 3 * (a + b + c) + 64;
   return bytes;
 }
 
