@@ -534,10 +534,10 @@ bool vl_admits(const trioseq_plan_s* plan, bool tb) {
 // triplet per register (wavefront_vl.cuh; build_batch falls back to int32 where the scheme or the
 // budget does not admit it), 16 x 64 tasks while they number at most two per SM (more warps than 32 x 64 tasks
 // give, each with a shorter step; beyond that their records cost more than they gain), else 32 x 64.
-// Measured, kernel time (16 x 64 / 32 x 64 / int32 default): score, protein, 300 residues (95 /
-// 50 tasks) 0.19 / 0.22 / 0.50 ms; 1,000 residues (1,008 / 512) 0.80 / 0.71 / 1.74 ms; traceback, DNA, 128
-// residues (16 / 8) 0.094 / 0.119 / 0.129 ms, 1,000 residues 1.01 / 0.96 / 1.47 ms, 96 triplets of
-// 200..600 3.3 / 3.2 / 6.3 ms; 1,024 semi-global triplets of 100..300 4.8 / 4.3 / 7.2 ms.
+// Measured, kernel time (16 x 64 / 32 x 64 / int32 default): score, protein, 300 residues (95 / 50 tasks)
+// 0.185 / 0.209 / 0.50 ms; 1,000 residues (1,008 / 512) 0.77 / 0.66 / 1.74 ms; traceback, DNA, 128
+// residues (16 / 8) 0.090 / 0.109 / 0.129 ms, 1,000 residues 0.95 / 0.89 / 1.47 ms, 96 triplets of
+// 200..600 3.2 / 3.0 / 6.3 ms; 1,024 semi-global triplets of 100..300 4.6 / 4.0 / 7.2 ms.
 // Kept on int32: launches of at most 8 such tasks, where the launch itself is most of the time
 // (64 residues: 50 against 63 us), and score batches of exactly two triplets that cannot pack.
 Variant default_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n, bool tb) {

@@ -66,10 +66,15 @@ struct VlGeom {
 // bound the resident warps in steps of one: `blocks` CTAs per SM.
 // CS = 0 keeps the lane's sigma''(y,z) tile in registers; CS = 1 and 2 keep it and row-major profiles in
 // shared memory (10 and 9 warps per SM).
-template <int NJ, int NH, int CS>
+// Two warps per sub-partition all but saturate it (32 x 64 tasks without waits: a step per 0.34 us with
+// one, 0.27 with two, 0.26 with three); a ninth one per SM takes some slack out of a launch's waits
+// (protein 4,000 residues 17.5 -> 17.2 ms, DNA traceback 3,000 residues 10.9 -> 10.1 ms), but not
+// where it costs spills (semi-global 19.3 -> 19.9 ms).
+template <int NJ, int NH, int CS, int AT = kGlobal>
 struct VlLaunch {
   static constexpr int warps = CS == 1 ? 2 : 1;
-  static constexpr int blocks = CS == 1 ? 5 : (CS == 2 ? 9 : (NH >= 8 ? 8 : (NJ >= 8 ? 8 : 12)));
+  static constexpr int blocks =
+      CS == 1 ? 5 : (CS == 2 ? 9 : (NH >= 8 ? 8 : (NJ >= 8 ? (AT == kSemiGlobal ? 8 : 9) : 12)));
   static constexpr int regs = 65536 / (warps * 32 * blocks) / 8 * 8;
   static constexpr int max_regs = regs > 255 ? 255 : regs;
 };
@@ -197,15 +202,17 @@ __device__ __forceinline__ void ld_halves(const unsigned short* p, unsigned (&v)
 // counts published every 8 steps, same kernel: protein, 300 residues, 0.52 -> 0.25 ms; local, 1,500
 // residues, 4.3 -> 1.9 ms; DNA traceback, 3,000 residues, 17.5 -> 14.5 ms.
 // Measured (kernel time, this form against the int32 tiles or the earlier two-per-register kernel that
-// kept absolute records by slice): DNA traceback, 1,000 residues, 1.45 -> 0.96 ms, 3,000 residues 21.7 ->
-// 11.1 ms, 96 triplets of 200..600 6.2 -> 3.2 ms; protein score, 300 residues, 0.50 -> 0.19 ms, 1,000
-// residues 1.74 -> 0.71 ms, 4,000 residues 28.0 (int32) and 21.7 -> 18.2 ms (3,520 GCUPS).
-// A lone warp's step of 32 x 64 cells takes 0.35 us (0.61 before) in ~370 instructions, of which 230 are
-// cell work at 2 cycles each on the ALU or the FMA pipe; the rest of a launch is waiting: the chain of
-// column tasks, and co-resident warps.
+// kept absolute records by slice): DNA traceback, 1,000 residues, 1.45 -> 0.90 ms, 3,000 residues 21.7 ->
+// 10.1 ms, 96 triplets of 200..600 6.2 -> 3.0 ms; protein score, 300 residues, 0.50 -> 0.19 ms, 1,000
+// residues 1.74 -> 0.67 ms, 4,000 residues 28.0 (int32) and 21.7 -> 17.2 ms (3,720 GCUPS).
+// A lone warp's step of 32 x 64 cells takes 0.34 us (0.61 before) in ~340 instructions, of which 200 are
+// cell work at 2 cycles each on the ALU or the FMA pipe. Mixed, the two pipes do not reach 2 x 64
+// instructions per SM and clock: three-register operands leave 85 (3-input max with a multiply-add) to
+// 103 (add-max with one), so operand reads bind a full sub-partition; the rest of a launch is the
+// chain of column tasks.
 template <int NJ, int NH, int CS, int AT, bool TB>
-__global__ void __launch_bounds__(VlLaunch<NJ, NH, CS>::warps * 32)
-    __maxnreg__((VlLaunch<NJ, NH, CS>::max_regs)) wavefront_vl_kernel(const WaveParams p) {
+__global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
+    __maxnreg__((VlLaunch<NJ, NH, CS, AT>::max_regs)) wavefront_vl_kernel(const WaveParams p) {
   static_assert(AT == kGlobal || CS == 0, "the variant types keep sigma'' in registers");
   static_assert(!TB || (AT == kGlobal && CS == 0 && NH == 4), "traceback keys: global, NH = 4");
   using G = VlGeom<NJ, NH>;
@@ -658,34 +665,33 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS>::warps * 32)
         int Bd[NH];  // sigma''(x, z) in the diagonal sum: without the rank offset of the 101 move
 #pragma unroll
         for (int qq = 0; qq < NH; ++qq) Bd[qq] = Bq[qq] - kOffK * 0x10001;
-        // The moves from the previous slice (E) one anti-diagonal ahead of the moves within the slice
-        // (Q): E's adds are FMA-pipe work, Q's maxima ALU-pipe work on a dependent chain, so each fills
-        // the other's waits. ea[pp] holds A + (row above, slice s - 1) of the last column done in row
-        // pp: the 110 sum of that column and the diagonal sum of the next.
-        int E[NJ][NH], Q[NJ][NH], ea[NJ];
+        // Q = max{ max(Pd + A + B, Myz) + C, Pxy + A, Pxz + B, Sx, Sy, Sz }: the diagonal and the (0,1,1)
+        // move share the add of C, so a register takes 4 ALU-pipe instructions (two fused add-maxima,
+        // two 3-input maxima) and 2.25 multiply-adds. (With E = max{ Pd + A + B + C, ... } formed first,
+        // 3.25: both pipes and the register reads bind, an SMSP does a step per 0.30 us at best.)
+        // The part from the previous slice (E, X) runs one anti-diagonal ahead of the part within the
+        // slice, so each fills the other's waits. ea[pp] holds A + (row above, slice s - 1) of the last
+        // column done in row pp: the 110 sum of that column and the diagonal sum of the next.
+        int E[NJ][NH], X[NJ][NH], Q[NJ][NH], ea[NJ];
 #pragma unroll
         for (int pp = 0; pp < NJ; ++pp)
           ea[pp] = mad_lo(A[pp], p.one, pp == 0 ? rowPrev[0] : colPrev[pp - 1]);
         auto from_prev = [&](const int pp, const int qq) {
           const int Pxy = (pp == 0) ? rowPrev[qq + 1] : P[pp - 1][qq];
           const int Pxz = (qq == 0) ? colPrev[pp] : P[pp][qq - 1];
-          const unsigned x2 = (unsigned)mad_lo(Bd[qq], p.one, ea[pp]);
+          X[pp][qq] = ea[pp];
           ea[pp] = mad_lo(A[pp], p.one, Pxy);
           const unsigned eb = (unsigned)mad_lo(Bq[qq], p.one, Pxz);
-          const unsigned e = __vimax3_u16x2((unsigned)ea[pp], eb, (unsigned)P[pp][qq]);
-          if constexpr (AT == kLocal) {
-            // v = 0: the diagonal's floor as the third input of one max, with x2 + C on the FMA pipe
-            const unsigned x2c = (unsigned)mad_lo((int)cv(pp, qq), p.one, (int)x2);
-            E[pp][qq] = (int)__vimax3_u16x2(x2c, e, fl);
-          } else {
-            E[pp][qq] = (int)__viaddmax_u16x2(x2, cv(pp, qq), e);
-          }
+          unsigned Sx = (unsigned)P[pp][qq];
+          if constexpr (AT == kLocal) Sx = __vmaxu2(Sx, fl);  // v = 0: the diagonal's floor
+          E[pp][qq] = (int)__vimax3_u16x2((unsigned)ea[pp], eb, Sx);
         };
         auto in_slice = [&](const int pp, const int qq) {
           const int Myz = (pp == 0) ? rowCur[qq] : (qq == 0 ? colCur[pp - 1] : Q[pp - 1][qq - 1]);
           const int Sy = (pp == 0) ? rowCur[qq + 1] : Q[pp - 1][qq];
           const int Sz = (qq == 0) ? colCur[pp] : Q[pp][qq - 1];
-          unsigned q = __viaddmax_u16x2((unsigned)Myz, cv(pp, qq), (unsigned)E[pp][qq]);
+          const unsigned w = __viaddmax_u16x2((unsigned)X[pp][qq], (unsigned)Bd[qq], (unsigned)Myz);
+          unsigned q = __viaddmax_u16x2(w, cv(pp, qq), (unsigned)E[pp][qq]);
           if constexpr (TB) {
             q = __viaddmax_u16x2((unsigned)Sy, 0xffffffffu, q);  // rank 2
             q = __viaddmax_u16x2((unsigned)Sz, 0xfffefffeu, q);  // rank 1
