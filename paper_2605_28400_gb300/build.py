@@ -38,6 +38,7 @@ def _inputs():
     files += [os.path.join(CSRC, "engine.h"), os.path.join(CSRC, "wavefront.cuh"),
               os.path.join(CSRC, "guard.h"),
               os.path.join(CSRC, "wavefront_vl.cuh"),
+              os.path.join(CSRC, "wavefront_vp.cuh"),
               os.path.join(ROOT, "include", "trioseq.h")]
     return files
 

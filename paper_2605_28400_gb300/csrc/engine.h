@@ -71,6 +71,9 @@ __host__ __device__ inline int vl_code_bit(int e) { return 16 * ((e >> 2) & 1) +
 // T rows of vl_rec_j(NH) and kVlRecK int32 per column task.
 constexpr int vl_rec_j(int NH) { return kPC * (NH + 2); }
 constexpr int kVlRecK = kPR * 6;
+// The two-triplets-per-register kernel (wavefront_vp.cuh): T rows of its words.
+constexpr int vp_rec_j(int NK) { return kPC * (NK + 1); }
+constexpr int vp_rec_k(int NJ) { return kPR * NJ; }
 
 struct TripDesc {
   int64_t s_off[3];    // byte offsets of S0, S1, S2 in the packed residue buffer
@@ -213,8 +216,10 @@ int wavefront_occupancy(int nj, int nk, bool tb, int at, int pk, bool slab, size
                         int* blocks_per_sm);
 // Kernel entry of a semi-global or local instantiation (kernels_variants.cu), or null.
 const void* wavefront_variant(int nj, int nk, int at, bool tb);
-// Kernel entry of a packed int16x2 (global, score) instantiation (kernels_packed.cu), or null.
+// Kernel entry of a packed int16x2 (global, score) instantiation (kernels_packed.cu), or null: mode 1
+// signed halves (wavefront.cuh), 2 biased halves (wavefront_vp.cuh).
 const void* wavefront_packed(int nj, int nk, int mode);
+size_t wavefront_vp_smem_bytes(int nj, int nk, int KP);
 // two cells of one triplet per register (wavefront_vl.cuh): nj x nk = 8 x 16, 8 x 8 or 4 x 8 cells
 // per lane; cs = 1 or 2: the lane's sigma''(y,z) tile in shared memory (8 x 16 only; 2-warp or
 // 1-warp CTAs), 0: in registers
@@ -228,7 +233,7 @@ int wavefront_vl_warps(int cs);
 const void* wavefront_slab(int nj, int nk, bool tb);
 int launch_walk(const WalkParams& p, void* stream);
 size_t wavefront_smem_bytes(int nj, int nk, int KP, bool pk);
-// threads per CTA of a launch in packed mode pk (1 warp for pk = 3 and 5, 2 for pk = 4, else
+// threads per CTA of a launch in packed mode pk (1 warp for pk = 2, 3 and 5, 2 for pk = 4, else
 // kWarpsPerCta)
 int wavefront_block_threads(int pk);
 

@@ -264,7 +264,7 @@ const void* pick(int nj, int nk, bool tb, int at, int pk, bool slab) {
 }  // namespace
 
 int wavefront_block_threads(int pk) {
-  return 32 * (pk >= 3 ? wavefront_vl_warps(pk - 3) : kWarpsPerCta);
+  return 32 * (pk >= 3 ? wavefront_vl_warps(pk - 3) : (pk == 2 ? 1 : kWarpsPerCta));
 }
 
 size_t wavefront_smem_bytes(int nj, int nk, int KP, bool pk) {

@@ -548,6 +548,24 @@ Variant default_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip,
   return tasks <= 2 * (uint64_t)plan->sms ? Variant{4, 8, 1} : Variant{8, 8, 1};
 }
 
+// The tile of a batch of pairs (two triplets per register, biased; wavefront_vp.cuh). 8x4 (32 x 32 tasks)
+// has the fewest instructions per cell that fit the registers; 4x4 (16 x 32) is 7% slower per cell, and
+// taken where its tasks pad less than that (lengths of a few tens), or where 8x4 would leave warps idle (at
+// most two tasks per SM). Kernel time, 8x4 / 4x8 / 4x4 / 8x8: 4,096 DNA triplets of 100..300 residues
+// 11.2 / 11.8 / 12.2 / 13.3 ms, of 30..60 260 / 243 / 243 / 350 us; 100 of 60..100 77 / 78 / 82 / 129 us; 8 of
+// 100..200 132 / 138 / 115 / 223 us; 300 protein triplets of 100..200 436 / 460 / 440 / 571 us.
+Variant packed_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n) {
+  double tasks = 0, wide = 0, narrow = 0;  // tasks of 8x4; padded cells of 8x4 and 4x4
+  for (size_t t = 0; t < n; t++) {
+    const double a = trip[t].len[0] + 11.0, k = (trip[t].len[2] + 32) / 32;
+    const double j8 = (trip[t].len[1] + 32) / 32, j4 = (trip[t].len[1] + 16) / 16;
+    tasks += 0.5 * j8 * k;
+    wide += a * j8 * k * 2;
+    narrow += a * j4 * k;
+  }
+  return tasks <= 2.0 * plan->sms || 1.08 * narrow < wide ? Variant{4, 4} : Variant{8, 4};
+}
+
 // Build the host side of a batch: encode, pack, describe, order the queue.
 trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n,
                            uint32_t mode, trioseq_batch_s* bt) {
@@ -574,9 +592,12 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
         bt->TI = it->second.TI;
       } else if (auto_tile(plan, tb) &&
                  !(n == 1 && plan->atype == kGlobal && plan->slab_slices > 0)) {
-        // global score batches whose pairs fit run two triplets per register on the int32 tile
-        if (!tb && plan->atype == kGlobal && n >= 2 && maxlen <= (1u << 24))
-          units = pack_units(plan, trip, n, kPR * bt->var.nj, kPC * bt->var.nk);
+        // global score batches whose pairs fit run two triplets per register
+        if (!tb && plan->atype == kGlobal && n >= 2 && maxlen <= (1u << 24)) {
+          const Variant v = plan->sig2_nonneg ? packed_variant(plan, trip, n) : bt->var;
+          units = pack_units(plan, trip, n, kPR * v.nj, kPC * v.nk);
+          if (!units.empty()) bt->var = v;
+        }
         if (units.empty()) bt->var = default_variant(plan, trip, n, tb);
       }
     }
@@ -735,12 +756,14 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
     d.T = a + 1 + (kPR - 1) + (kPC - 1) + (vl ? kPC : 0);  // vl: 2*kPC virtual lane columns
     // boundary records of every column task: (a+1) x (WK+4) j-records, (a+1) x WJ k-records
     const size_t ntask = (size_t)d.nJ * (size_t)d.nK;
-    // (vl: by producer step, T x vl_rec_j and T x kVlRecK)
+    // (two per register, biased: by producer step, T rows)
+    const bool by_step = vl || bt->packed == 2;
     d.oj_off = (int64_t)face;
-    face += vl ? ntask * (size_t)d.T * (size_t)vl_rec_j(NK / 2)
-               : ntask * (size_t)(a + 1) * (size_t)(WK + 4);
+    face += by_step ? ntask * (size_t)d.T * (size_t)(vl ? vl_rec_j(NK / 2) : vp_rec_j(NK))
+                    : ntask * (size_t)(a + 1) * (size_t)(WK + 4);
     d.ok_off = (int64_t)face;
-    face += vl ? ntask * (size_t)d.T * (size_t)kVlRecK : ntask * (size_t)(a + 1) * (size_t)WJ;
+    face += by_step ? ntask * (size_t)d.T * (size_t)(vl ? kVlRecK : vp_rec_k(NJ))
+                    : ntask * (size_t)(a + 1) * (size_t)WJ;
     face = align_up(face, 4);
     d.prog_base = prog;
     prog += (int64_t)d.nJ * d.nK;
@@ -865,7 +888,8 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   layout_inputs(bt);
   // launch shape
   bt->smem = bt->packed >= 3 ? wavefront_vl_smem_bytes(NJ, NK, plan->KP, bt->packed - 3)
-                             : wavefront_smem_bytes(NJ, NK, plan->KP, bt->packed != 0);
+             : bt->packed == 2 ? wavefront_vp_smem_bytes(NJ, NK, plan->KP)
+                               : wavefront_smem_bytes(NJ, NK, plan->KP, bt->packed != 0);
   int bpm = 0;
   // Int32 traceback launches of one triplet use the records as readiness flags; TRIOSEQ_DATA_FLAGS at
   // plan creation forces it on (1) or off (0). (The two-cells-per-register kernel always does.)
@@ -876,7 +900,7 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
     return TRIOSEQ_ECUDA;
   const int want = env_int("TRIOSEQ_CTAS_PER_SM", bpm);
   bt->grid = plan->sms * std::max(1, std::min(bpm, want));
-  if (vl)  // no CTA without a task: one that finds the queue empty still costs its start
+  if (vl || bt->packed == 2)  // no CTA without a task: one that finds the queue empty still costs its start
     bt->grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)bt->grid, bt->tasks.size()));
   return TRIOSEQ_OK;
 }
@@ -1051,7 +1075,7 @@ trioseq_status run(trioseq_batch_s* bt, cudaStream_t st) {
     p.pace_n = bt->grid * warps_per_cta;
     p.pace_T = 1 << 20;
     p.pace_flag = prog + bt->tasks.size() + 48;
-  } else if (!bt->slab && plan->pace && !p.data_flags && bt->packed < 3 &&
+  } else if (!bt->slab && plan->pace && !p.data_flags && bt->packed < 2 &&
              bt->tasks.size() >= 2 * (size_t)bt->grid * warps_per_cta) {
     // pace the first wave against the progress of queue task 0, the (0,0) block of its triplet
     const TripDesc& d0 = bt->desc[bt->tasks[0].trip];
@@ -1588,10 +1612,12 @@ trioseq_status trioseq_batch_kernel(trioseq_batch_t bt, char* name, size_t cap) 
       std::snprintf(buf, sizeof buf, "wavefront_vl_kernel<%d,%d,%d%s> tile %dx%d%s", nj, nk / 2,
                     bt->packed - 3, tb ? ",traceback" : "", nj, nk,
                     bt->packed == 4 ? "s" : (bt->packed == 5 ? "t" : (nk == 16 ? "" : "v")));
+    else if (bt->packed == 2)
+      std::snprintf(buf, sizeof buf, "wavefront_vp_kernel<%d,%d> tile %dx%d", nj, nk, nj, nk);
     else if (bt->packed)
-      std::snprintf(buf, sizeof buf, "wavefront_kernel<%d,%d,score,global,%s> tile %dx%d", nj, nk,
-                    bt->packed == 2 ? "two triplets per register, biased" :
-                                      "two triplets per register, signed", nj, nk);
+      std::snprintf(buf, sizeof buf,
+                    "wavefront_kernel<%d,%d,score,global,two triplets per register, signed> tile %dx%d",
+                    nj, nk, nj, nk);
     else
       std::snprintf(buf, sizeof buf, "wavefront_kernel<%d,%d,%s,%s%s> tile %dx%d", nj, nk,
                     tb ? "traceback" : "score", type, bt->slab ? ",slab" : "", nj, nk);

@@ -421,6 +421,7 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
         if (ok && has_k) ok = wait_flag(prog - 1, 1, &seen, p.wait_ns);
       }
       ok = __shfl_sync(kFull, ok, 0);
+      __syncwarp();  // the other lanes' loads come after lane 0's acquire
     }
 
     // A piece: the words and (corner, base) or (base, base) of one item in pair u (steps u and u + 1,
