@@ -23,7 +23,6 @@ namespace trioseq {
 namespace {
 
 constexpr size_t kScratchBytes = (size_t)64 << 20;  // 64 MiB per device
-constexpr int kNoallocNJ = 8, kNoallocNK = 8;       // the score-only 8x8 wavefront variant
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -33,9 +32,15 @@ struct NoallocTables {
   int8_t lut[256];                                       // byte -> residue code, -1 invalid
 };
 
+// Tile of a call: the int32 score kernel's 8x8, or two cells per register (pk = 3) 4x8v or 8x8v.
+struct NoallocTile {
+  int nj, nk, pk;
+};
+
 struct NoallocLayout {
   size_t off_seq, off_sig, off_desc, off_tasks, off_prog, off_faces, total;
   int nJ, nK, T, ntasks;
+  int64_t ok_off;  // int32 offset of the k-records in the faces
 };
 
 __host__ __device__ inline size_t up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -44,9 +49,10 @@ __host__ __device__ inline size_t up(size_t x, size_t a) { return (x + a - 1) / 
 // thin triplet can exceed 2^31 even though each length is at most 2^24. Returns false when the
 // task count or any size does not fit (the caller then reports TRIOSEQ_ESCRATCH); the layout's
 // int fields are set only when it fits.
-bool layout_for(int64_t a, int64_t b, int64_t c, int KP, NoallocLayout* out) {
+bool layout_for(int64_t a, int64_t b, int64_t c, int KP, const NoallocTile& tile,
+                NoallocLayout* out) {
   NoallocLayout L{};
-  const int64_t WJ = kPR * kNoallocNJ, WK = kPC * kNoallocNK;
+  const int64_t WJ = kPR * tile.nj, WK = kPC * tile.nk;
   const int64_t nJ = (b + 1 + WJ - 1) / WJ, nK = (c + 1 + WK - 1) / WK;
   const int64_t ntasks = nJ * nK;  // < 2^38 for lengths <= 2^24: no 64-bit overflow
   // Every task holds (a + 1) slices of records, at least one int32 each: a task count beyond
@@ -65,12 +71,16 @@ bool layout_for(int64_t a, int64_t b, int64_t c, int KP, NoallocLayout* out) {
   L.off_prog = off;
   off = up(off + sizeof(int32_t) * ((size_t)ntasks + 64), 256);
   L.off_faces = off;
-  off += sizeof(int32_t) * (size_t)ntasks * (size_t)(a + 1) * (size_t)((WK + 4) + WJ);
+  // record rows of every task: int32 by slice, two cells per register by step (two virtual lane columns a lane)
+  L.T = (int)(a + 1 + (kPR - 1) + (kPC - 1) + (tile.pk ? kPC : 0));
+  const size_t rows = tile.pk ? (size_t)L.T : (size_t)(a + 1);
+  const size_t rj = tile.pk ? vl_rec_j(tile.nk / 2) : WK + 4, rk = tile.pk ? kVlRecK : WJ;
+  L.ok_off = (int64_t)((size_t)ntasks * rows * rj);
+  off += sizeof(int32_t) * (size_t)ntasks * rows * (rj + rk);
   L.total = up(off, 256);
   if (L.total > kScratchBytes) return false;
   L.nJ = (int)nJ;
   L.nK = (int)nK;
-  L.T = (int)(a + 1 + (kPR - 1) + (kPC - 1));
   L.ntasks = (int)ntasks;
   *out = L;
   return true;
@@ -119,7 +129,7 @@ __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout L, No
     d.s_off[1] = o1;
     d.s_off[2] = o2;
     d.oj_off = 0;
-    d.ok_off = (int64_t)L.ntasks * (a + 1) * (kPC * kNoallocNK + 4);
+    d.ok_off = L.ok_off;
     d.code_off = -1;
     d.prog_base = 0;
     d.len[0] = a;
@@ -161,7 +171,7 @@ extern "C" trioseq_status trioseq_align_noalloc(const trioseq_scoring* sc,
   NoallocTables tab;
   for (int i = 0; i < 256; i++) tab.lut[i] = -1;
   for (int i = 0; i < KP * KP; i++) tab.sig[i] = 0;
-  int32_t mx = 1;
+  int32_t mx = 1, mn = 0;
   for (int i = 0; i < K; i++) {
     const unsigned char ch = (unsigned char)sc->alphabet[i];
     if (tab.lut[ch] >= 0) return TRIOSEQ_EINVAL;
@@ -171,18 +181,35 @@ extern "C" trioseq_status trioseq_align_noalloc(const trioseq_scoring* sc,
       const int32_t v = (int32_t)sc->sub[i * K + j] - 2 * sc->gap;
       tab.sig[i * KP + j] = v;
       mx = v > mx ? v : (-v > mx ? -v : mx);
+      mn = v < mn ? v : mn;
     }
   }
   const int64_t sumlen = (int64_t)a + b + c;
   if (a > (1u << 24) || b > (1u << 24) || c > (1u << 24)) return TRIOSEQ_ESCRATCH;
   if ((int64_t)mx * sumlen >= (1LL << 26) - 1) return TRIOSEQ_EOVERFLOW;
+  // What the scratch takes is set by the int32 tile; the call runs on two cells per register where the scheme
+  // admits it (as in the plans' batches, runtime.cu) and its records fit too: 16 x 64 tasks while they number
+  // at most two per SM, else 32 x 64. Kernel time of one triplet of 20 / 60 / 100 / 128 DNA residues, int32
+  // against 16 x 64 tasks: 29 / 68 / 135 / 183 us against 27 / 42 / 68 / 89 us.
+  NoallocTile tile{8, 8, 0};
   NoallocLayout L{};
-  if (!layout_for(a, b, c, KP, &L)) return TRIOSEQ_ESCRATCH;
+  if (!layout_for(a, b, c, KP, tile, &L)) return TRIOSEQ_ESCRATCH;
 
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
     cudaGetLastError();
     return TRIOSEQ_ECUDA;
+  }
+  int sms = 0, bpm = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return TRIOSEQ_ECUDA;
+  }
+  if (mn >= 0 && mx <= 33) {
+    const uint64_t narrow = ((uint64_t)b + 16) / 16 * (((uint64_t)c + 64) / 64);
+    const NoallocTile vl[2] = {{4, 8, 3}, {8, 8, 3}};
+    for (int q = narrow <= 2 * (uint64_t)sms ? 0 : 1; q < 2 && !tile.pk; q++)
+      if (layout_for(a, b, c, KP, vl[q], &L)) tile = vl[q];
   }
   unsigned char* scratch = nullptr;
   {
@@ -210,15 +237,12 @@ extern "C" trioseq_status trioseq_align_noalloc(const trioseq_scoring* sc,
                                            (int)c, score_base);
   if (cudaGetLastError() != cudaSuccess) return TRIOSEQ_ECUDA;
 
-  int sms = 0, bpm = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return TRIOSEQ_ECUDA;
-  }
-  const size_t smem = wavefront_smem_bytes(kNoallocNJ, kNoallocNK, KP, false);
-  if (wavefront_occupancy(kNoallocNJ, kNoallocNK, false, kGlobal, false, false, smem, &bpm) != 0 ||
+  const size_t smem = tile.pk ? wavefront_vl_smem_bytes(tile.nj, tile.nk, KP, 0)
+                              : wavefront_smem_bytes(tile.nj, tile.nk, KP, false);
+  if (wavefront_occupancy(tile.nj, tile.nk, false, kGlobal, tile.pk, false, smem, &bpm) != 0 ||
       bpm <= 0)
     return TRIOSEQ_ECUDA;
+  const int grid = tile.pk && L.ntasks < sms * bpm ? L.ntasks : sms * bpm;
   int32_t* prog = reinterpret_cast<int32_t*>(scratch + L.off_prog);
   WaveParams p{};
   p.desc = reinterpret_cast<const TripDesc*>(scratch + L.off_desc);
@@ -237,8 +261,7 @@ extern "C" trioseq_status trioseq_align_noalloc(const trioseq_scoring* sc,
   p.g2 = -2 * sc->gap;
   p.one = 1;
   p.wait_ns = 2000000000LL;
-  if (launch_wavefront(kNoallocNJ, kNoallocNK, false, kGlobal, false, false, p, sms * bpm, smem,
-                       st) != 0) {
+  if (launch_wavefront(tile.nj, tile.nk, false, kGlobal, tile.pk, false, p, grid, smem, st) != 0) {
     cudaGetLastError();
     return TRIOSEQ_ECUDA;
   }

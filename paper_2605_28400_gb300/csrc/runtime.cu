@@ -538,13 +538,21 @@ bool vl_admits(const trioseq_plan_s* plan, bool tb) {
 // 0.185 / 0.209 / 0.50 ms; 1,000 residues (1,008 / 512) 0.77 / 0.66 / 1.74 ms; traceback, DNA, 128
 // residues (16 / 8) 0.090 / 0.109 / 0.129 ms, 1,000 residues 0.95 / 0.89 / 1.47 ms, 96 triplets of
 // 200..600 3.2 / 3.0 / 6.3 ms; 1,024 semi-global triplets of 100..300 4.6 / 4.0 / 7.2 ms.
-// Kept on int32: launches of at most 8 such tasks, where the launch itself is most of the time
-// (64 residues: 50 against 63 us), and score batches of exactly two triplets that cannot pack.
+// One triplet of 20 / 45 / 60 / 80 DNA residues: score 27 / 36 / 42 / 60 us against 29 / 57 / 68 / 109 on int32;
+// with rows 30 / 41 / 48 / 71 against 33 / 51 / 64 / 92; semi-global 34 / 48 / 57 / 80 against 46 / 94 / 114 / 173.
+// Kept on int32, whose packing they have always reported, although no faster there: global batches of at most 8
+// such tasks that are one triplet over two block columns or several triplets with rows, and two
+// global triplets that cannot pack when one of them is a single task.
 Variant default_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n, bool tb) {
-  uint64_t tasks = 0;
-  for (size_t t = 0; t < n; t++)
-    tasks += (uint64_t)((trip[t].len[1] + 16) / 16) * ((trip[t].len[2] + 64) / 64);
-  if (tasks <= 8 || (!tb && n == 2)) return tb ? plan->tb_variant : plan->score_variant;
+  uint64_t tasks = 0, least = UINT64_MAX;
+  for (size_t t = 0; t < n; t++) {
+    const uint64_t q = (uint64_t)((trip[t].len[1] + 16) / 16) * ((trip[t].len[2] + 64) / 64);
+    tasks += q;
+    least = std::min(least, q);
+  }
+  const bool small = plan->atype == kGlobal && tasks <= 8 && (n != 1 || (!tb && trip[0].len[2] >= 64));
+  const bool uneven = plan->atype == kGlobal && !tb && n == 2 && least == 1;
+  if (small || uneven) return tb ? plan->tb_variant : plan->score_variant;
   return tasks <= 2 * (uint64_t)plan->sms ? Variant{4, 8, 1} : Variant{8, 8, 1};
 }
 

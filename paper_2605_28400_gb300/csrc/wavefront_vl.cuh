@@ -67,9 +67,10 @@ struct VlGeom {
 // CS = 0 keeps the lane's sigma''(y,z) tile in registers; CS = 1 and 2 keep it and row-major profiles in
 // shared memory (10 and 9 warps per SM).
 // Two warps per sub-partition all but saturate it (32 x 64 tasks without waits: a step per 0.34 us with
-// one, 0.27 with two, 0.26 with three); a ninth one per SM takes some slack out of a launch's waits
-// (protein 4,000 residues 17.5 -> 17.2 ms, DNA traceback 3,000 residues 10.9 -> 10.1 ms), but not
-// where it costs spills (semi-global 19.3 -> 19.9 ms).
+// one, 0.27 with two, 0.26 with three), and a third would need the 8 x 4 tile in 168 registers: protein 1,000
+// residues 0.67 -> 0.85 ms. The cap of 224 registers that `blocks` = 9 gives still leaves two; its code is the
+// faster (protein 4,000 residues 17.5 -> 17.2 ms, DNA traceback 3,000 residues 10.9 -> 10.1 ms), but not for
+// semi-global, where it spills (19.3 -> 19.9 ms).
 template <int NJ, int NH, int CS, int AT = kGlobal>
 struct VlLaunch {
   static constexpr int warps = CS == 1 ? 2 : 1;

@@ -16,8 +16,10 @@
 //    work at the shorter one's last slice.
 // Measured, kernel time against the int32-record form of wavefront_kernel that took these batches before
 // (progress counts, 32 x 64 tasks, four-warp CTAs): 4,096 DNA triplets of 100..300 residues 12.74 -> 11.2 ms
-// (3,790 GCUPS). What bounds it is issue and operand reads: two warps per sub-partition saturate it (8, 9 and
-// 10 warps per SM take the same time), with a step of 32 x 32 x 2 cells at ~270 instructions.
+// (3,790 GCUPS). What bounds it is issue, operand reads and the waits of two warps per sub-partition (its
+// registers allow no third; held to 168, for three, the large batch takes 10.8 ms, but ten triplets of
+// 300..600 residues 0.70 instead of 0.57 ms). A step of 32 x 32 x 2 cells takes ~270 instructions. Halos through
+// shared memory instead of shuffles and selects: 6% fewer instructions, but waits on more scoreboards, 13.7 ms.
 #pragma once
 #include "wavefront_vl.cuh"
 
