@@ -764,13 +764,13 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
     d.T = a + 1 + (kPR - 1) + (kPC - 1) + (vl ? kPC : 0);  // vl: 2*kPC virtual lane columns
     // boundary records of every column task: (a+1) x (WK+4) j-records, (a+1) x WJ k-records
     const size_t ntask = (size_t)d.nJ * (size_t)d.nK;
-    // (two per register, biased: by producer step, T rows)
+    // (two per register, biased: T rows by producer step, of the tasks that have a consumer)
     const bool by_step = vl || bt->packed == 2;
     d.oj_off = (int64_t)face;
-    face += by_step ? ntask * (size_t)d.T * (size_t)(vl ? vl_rec_j(NK / 2) : vp_rec_j(NK))
+    face += by_step ? (ntask - d.nK) * (size_t)d.T * (size_t)(vl ? vl_rec_j(NK / 2) : vp_rec_j(NK))
                     : ntask * (size_t)(a + 1) * (size_t)(WK + 4);
     d.ok_off = (int64_t)face;
-    face += by_step ? ntask * (size_t)d.T * (size_t)(vl ? kVlRecK : vp_rec_k(NJ))
+    face += by_step ? (ntask - d.nJ) * (size_t)d.T * (size_t)(vl ? kVlRecK : vp_rec_k(NJ))
                     : ntask * (size_t)(a + 1) * (size_t)WJ;
     face = align_up(face, 4);
     d.prog_base = prog;

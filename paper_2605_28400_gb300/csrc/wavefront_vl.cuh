@@ -290,7 +290,9 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
     const int8_t* S1 = p.seq + d.s_off[1];
     const int8_t* S2 = p.seq + d.s_off[2];
     const int j0 = J * WJ + r * NJ, k0 = K * WK + lc * NK;
-    const int me = J * nK + K;
+    // records exist where there is a consumer: j-rows of all but the last block row, k-rows of all but the
+    // last block column
+    const int me = J * nK + K, mek = J * (nK - 1) + K;
 
     // Profiles of this block: sigma''(x, y_j) and sigma''(x, z_k); residue index 0 and beyond the
     // end are VIRT.
@@ -395,11 +397,11 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
     const int it_stride = is_j ? G::RJ : G::RK;
     const int* it_src =
         p.faces + (is_j ? d.oj_off + ((int64_t)(me - nK) * T + (kPR - 1) + g) * G::RJ
-                        : d.ok_off + ((int64_t)(me - 1) * T + (2 * kPC - 1) + g) * G::RK);
+                        : d.ok_off + ((int64_t)(mek - 1) * T + (2 * kPC - 1) + g) * G::RK);
     const bool out_j = r == kPR - 1 && J + 1 < nJ, out_k = lc == kPC - 1 && K + 1 < nK;
     const int f_oj = vl_flag(out_j), f_ok = vl_flag(out_k);
     int* dstJ = p.faces + d.oj_off + (int64_t)me * T * G::RJ + lc * NH;
-    int* dstK = p.faces + d.ok_off + (int64_t)me * T * G::RK + r * 4;
+    int* dstK = p.faces + d.ok_off + (int64_t)mek * T * G::RK + r * 4;
     bool ok = true;
     uint32_t* codes = TB ? p.codes + d.code_off + (int64_t)me * T * 32 * W + lane * W : nullptr;
     // Without a producer the halo of the first lane row or column stays -infinity.
@@ -412,7 +414,7 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
           st_relaxed_if(q4 + e, make_int4(kVlSentinel, kVlSentinel, kVlSentinel, kVlSentinel), true);
       };
       if (J + 1 < nJ) fill(p.faces + d.oj_off + (int64_t)me * T * G::RJ, (int64_t)T * G::RJ);
-      if (K + 1 < nK) fill(p.faces + d.ok_off + (int64_t)me * T * G::RK, (int64_t)T * G::RK);
+      if (K + 1 < nK) fill(p.faces + d.ok_off + (int64_t)mek * T * G::RK, (int64_t)T * G::RK);
       __syncwarp();
       int* prog = p.progress + d.prog_base + me;
       if (lane == 0) {

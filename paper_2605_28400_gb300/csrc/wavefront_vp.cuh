@@ -108,7 +108,9 @@ __global__ void __launch_bounds__(32) __maxnreg__((VpLaunch<NJ, NK>::max_regs))
     const int8_t* S0 = p.seq + d.s_off[0];
     const int8_t* T0 = p.seq + d1.s_off[0];
     const int j0 = J * WJ + r * NJ, k0 = K * WK + lc * NK;
-    const int me = J * nK + K;
+    // records exist where there is a consumer: j-rows of all but the last block row, k-rows of all but the
+    // last block column
+    const int me = J * nK + K, mek = J * (nK - 1) + K;
 
     // Profiles of this block for both triplets: sigma''(x, y_j) and sigma''(x, z_k); residue index 0 and
     // beyond the end are VIRT.
@@ -196,10 +198,10 @@ __global__ void __launch_bounds__(32) __maxnreg__((VpLaunch<NJ, NK>::max_regs))
     const int it_stride = is_j ? G::RJ : G::RK;
     const int* it_src =
         p.faces + (is_j ? d.oj_off + ((int64_t)(me - nK) * T + (kPR - 1) + g) * G::RJ
-                        : d.ok_off + ((int64_t)(me - 1) * T + (kPC - 1) + g) * G::RK);
+                        : d.ok_off + ((int64_t)(mek - 1) * T + (kPC - 1) + g) * G::RK);
     const int f_oj = vl_flag(r == kPR - 1 && J + 1 < nJ), f_ok = vl_flag(lc == kPC - 1 && K + 1 < nK);
     int* dstJ = p.faces + d.oj_off + (int64_t)me * T * G::RJ + lc * NK;
-    int* dstK = p.faces + d.ok_off + (int64_t)me * T * G::RK + r * NJ;
+    int* dstK = p.faces + d.ok_off + (int64_t)mek * T * G::RK + r * NJ;
     bool ok = true;
     // Without a producer the halo of the first lane row or column stays -infinity.
     for (int e = lane; e < kRing * G::SLOT; e += 32) ring[e] = 0;
@@ -211,7 +213,7 @@ __global__ void __launch_bounds__(32) __maxnreg__((VpLaunch<NJ, NK>::max_regs))
           st_relaxed_if(q4 + e, make_int4(kVlSentinel, kVlSentinel, kVlSentinel, kVlSentinel), true);
       };
       if (J + 1 < nJ) fill(p.faces + d.oj_off + (int64_t)me * T * G::RJ, (int64_t)T * G::RJ);
-      if (K + 1 < nK) fill(p.faces + d.ok_off + (int64_t)me * T * G::RK, (int64_t)T * G::RK);
+      if (K + 1 < nK) fill(p.faces + d.ok_off + (int64_t)mek * T * G::RK, (int64_t)T * G::RK);
       __syncwarp();
       int* prog = p.progress + d.prog_base + me;
       if (lane == 0) {
