@@ -182,8 +182,16 @@ def _triplet_array(triplets):
     into it, so marshalling thousands of triplets costs one copy of the residues rather than one
     Python call per field. The library only reads the strings (it copies them before returning)."""
     n = len(triplets)
-    if any(len(t) != 3 for t in triplets):
+    if n and set(map(len, triplets)) != {3}:
         raise ValueError("a triplet has three sequences")
+    if n == 1:  # one record, without the arrays below
+        parts = triplets[0]
+        if all(isinstance(x, str) for x in parts):
+            parts = [x.encode("latin-1") for x in parts]
+        else:
+            parts = [_as_bytes(x) for x in parts]
+        rec = Triplet(tuple(parts), tuple(map(len, parts)))
+        return ctypes.pointer(rec), (parts, rec)
     flat = list(itertools.chain.from_iterable(triplets))
     try:  # all str (the common case): one join, one byte per character, as residues are
         joined = "".join(flat).encode("latin-1")
@@ -246,6 +254,11 @@ def trioseq_align_batch(plan, triplets, mode: int = SCORE_ONLY, stream=None) -> 
     return out[:len(triplets)]
 
 
+def _split_rows(buf, size: int, L: int):
+    raw = buf.tobytes()
+    return tuple(raw[q:q + L].decode() for q in (0, size, 2 * size))
+
+
 def _rows(fn, handle, idx: int, cap: int | None = None):
     lib = load()
     n = ctypes.c_size_t(0)
@@ -255,9 +268,14 @@ def _rows(fn, handle, idx: int, cap: int | None = None):
     if st != EINVAL or n.value == 0:
         _check(st, fn.__name__)
     cap = n.value if cap is None else cap
-    bufs = [ctypes.create_string_buffer(max(1, cap)) for _ in range(3)]
-    _check(fn(handle, idx, bufs[0], bufs[1], bufs[2], cap, ctypes.byref(n)), fn.__name__)
-    return tuple(b.raw[:n.value].decode() for b in bufs)
+    size = max(1, cap)
+    buf = np.empty(3 * size, dtype=np.uint8)  # the three rows one after another
+    base, char_p = buf.ctypes.data, ctypes.c_char_p
+    st = fn(handle, idx, char_p(base), char_p(base + size), char_p(base + 2 * size), cap,
+            ctypes.byref(n))
+    if st != OK:
+        _check(st, fn.__name__)
+    return _split_rows(buf, size, n.value)
 
 
 def trioseq_traceback(plan, idx: int, cap: int | None = None):
@@ -378,16 +396,17 @@ def trioseq_poll(server, ticket: int, cap: int = 0):
     score = ctypes.c_int32(0)
     n = ctypes.c_size_t(0)
     if cap > 0:
-        bufs = [ctypes.create_string_buffer(cap) for _ in range(3)]
-        rows = (ctypes.c_char_p * 3)(*[ctypes.cast(b, ctypes.c_char_p) for b in bufs])
+        buf = np.empty(3 * cap, dtype=np.uint8)  # the three rows one after another
+        base = buf.ctypes.data
+        rows = (ctypes.c_char_p * 3)(base, base + cap, base + 2 * cap)
     else:
-        bufs, rows = None, None
+        buf, rows = None, None
     st = load().trioseq_poll(server, ctypes.c_uint64(ticket), ctypes.byref(score), rows,
                              int(cap), ctypes.byref(n))
     if st == EAGAIN:
         return st, None, None
     _check(st, "trioseq_poll")
-    out_rows = tuple(b.raw[:n.value].decode() for b in bufs) if bufs and n.value else None
+    out_rows = _split_rows(buf, cap, n.value) if buf is not None and n.value else None
     return st, int(score.value), out_rows
 
 

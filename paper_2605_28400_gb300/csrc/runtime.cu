@@ -136,7 +136,7 @@ struct Workspace {
   DevBuf walkstate; // slab mode: (i, j, k, n) of the traceback walk between slabs
   DevBuf best64;    // semi-global / local traceback: (score, first cell) key per triplet
   DevBuf spans;     // traceback: begin and end cell of each alignment (6 int32)
-  HostPinned staging;
+  HostPinned staging, results;  // per-call path: inputs up, results down
   // Buffers are allocated and freed in this stream's order. Plans and device-resident batches
   // own a private stream here (own_stream); a serving slot uses its launch stream.
   cudaStream_t alloc_stream = nullptr;
@@ -499,14 +499,15 @@ std::vector<std::pair<int32_t, int32_t>> pack_units(const trioseq_plan_s* plan,
                                                     const trioseq_triplet* trip, size_t n, int WJ,
                                                     int WK) {
   std::vector<std::pair<int32_t, int32_t>> units;
-  std::vector<int32_t> order(n);
-  for (size_t t = 0; t < n; t++) order[t] = (int32_t)t;
-  const auto cls = [&](int32_t t) {
+  // by grid class, then length, then position (keys beside the indices: sorting reads no triplet)
+  std::vector<std::tuple<uint64_t, uint32_t, int32_t>> keys(n);
+  for (size_t t = 0; t < n; t++) {
     const uint32_t* L = trip[t].len;
-    return std::make_tuple((L[1] + WJ) / WJ, (L[2] + WK) / WK, L[0]);
-  };
-  std::stable_sort(order.begin(), order.end(),
-                   [&](int32_t x, int32_t y) { return cls(x) < cls(y); });
+    keys[t] = {(uint64_t)((L[1] + WJ) / WJ) << 32 | (L[2] + WK) / WK, L[0], (int32_t)t};
+  }
+  std::sort(keys.begin(), keys.end());
+  std::vector<int32_t> order(n);
+  for (size_t t = 0; t < n; t++) order[t] = std::get<2>(keys[t]);
   for (size_t u = 0; u < n; u += 2) {
     const int32_t t0 = order[u], t1 = (u + 1 < n) ? order[u + 1] : order[u];
     int64_t gsum = 0;
@@ -679,8 +680,11 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
           if (acc < 0) bad.store(true, std::memory_order_relaxed);
         }
     };
-    const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    const size_t nth = std::min<size_t>({(size_t)8, (size_t)hw, n, total / (1u << 19) + 1});
+    // a thread per 128 KiB of residues (~140 us of work); the thread count is asked for only then (it reads
+    // the system's files: 10 us, most of a small call's encoding)
+    size_t nth = std::min<size_t>({(size_t)8, n, total / (1u << 17) + 1});
+    if (nth > 1)
+      nth = std::min<size_t>(nth, std::max(1u, std::thread::hardware_concurrency()));
     if (nth <= 1) {
       encode(0, n);
     } else {  // split the triplets into nth ranges of about equal residue counts
@@ -863,14 +867,14 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   // a stable sort on the full key.
   const size_t nu = units.size();
   std::vector<int32_t> order(nu);
-  for (size_t u = 0; u < nu; u++) order[u] = (int32_t)u;
   {
-    const auto vol = [&](int32_t u) {
+    std::vector<std::pair<double, int32_t>> key(nu);  // largest volume first, then position
+    for (size_t u = 0; u < nu; u++) {
       const TripDesc& d = bt->desc[units[u].first];
-      return (double)(d.glen[0] + 1) * (d.glen[1] + 1) * (d.glen[2] + 1);
-    };
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int32_t x, int32_t y) { return vol(x) > vol(y); });
+      key[u] = {-(double)(d.glen[0] + 1) * (d.glen[1] + 1) * (d.glen[2] + 1), (int32_t)u};
+    }
+    std::sort(key.begin(), key.end());
+    for (size_t u = 0; u < nu; u++) order[u] = key[u].second;
   }
   int maxD = 0;
   for (const auto& un : units) {
@@ -1222,34 +1226,47 @@ trioseq_status run_graph(trioseq_batch_s* bt, cudaStream_t st) {
   return TRIOSEQ_OK;
 }
 
-// Wait for the run, check the error word, fetch scores (and traceback rows).
-trioseq_status fetch(trioseq_batch_s* bt, cudaStream_t st, int32_t* scores_out) {
+// Wait for the run, check the error word, fetch scores (and traceback rows). With `stage`, the copies go to
+// that pinned buffer, enqueued behind the run, and are handed on after one wait (a copy to pageable memory
+// holds the caller for its own round trip: 48 us for the five of a call with rows, 22 us for the two of a score
+// call, against 9 and 6); without, straight to their destinations, which several threads may do at once.
+trioseq_status fetch(trioseq_batch_s* bt, cudaStream_t st, int32_t* scores_out,
+                     HostPinned* stage = nullptr) {
   Workspace& ws = *bt->ws;
   const bool tb = bt->mode == TRIOSEQ_WITH_TRACEBACK;
   int32_t herr = 0;
   cudaError_t e = cudaSuccess;
+  struct Part {
+    void* dst;
+    const void* src;
+    size_t bytes, off;
+  };
+  Part parts[5];
+  int np = 0;
+  size_t total = 0;
+  const auto add = [&](void* dst, const void* src, size_t bytes) {
+    parts[np++] = Part{dst, src, bytes, total};
+    total += align_up(bytes, 64);
+  };
   if (bt->n) {
-    int32_t* err = ws.progress.as<int32_t>() + bt->tasks.size() + 32;
-    e = cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && scores_out)
-      e = cudaMemcpyAsync(scores_out, ws.scores.p, bt->n * sizeof(int32_t),
-                          cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && tb && !bt->tb_trips.empty()) {
+    add(&herr, ws.progress.as<int32_t>() + bt->tasks.size() + 32, sizeof(int32_t));
+    if (scores_out) add(scores_out, ws.scores.p, bt->n * sizeof(int32_t));
+    if (tb && !bt->tb_trips.empty()) {
       bt->h_rows.resize(bt->rows_bytes);
       bt->h_lens.resize(bt->tb_trips.size());
-      e = cudaMemcpyAsync(bt->h_rows.data(), ws.rows.p, bt->rows_bytes, cudaMemcpyDeviceToHost,
-                          st);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(bt->h_lens.data(), ws.lens.p, bt->h_lens.size() * sizeof(int32_t),
-                            cudaMemcpyDeviceToHost, st);
       bt->h_spans.resize(6 * bt->tb_trips.size());
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(bt->h_spans.data(), ws.spans.p, bt->h_spans.size() * sizeof(int32_t),
-                            cudaMemcpyDeviceToHost, st);
+      add(bt->h_rows.data(), ws.rows.p, bt->rows_bytes);
+      add(bt->h_lens.data(), ws.lens.p, bt->h_lens.size() * sizeof(int32_t));
+      add(bt->h_spans.data(), ws.spans.p, bt->h_spans.size() * sizeof(int32_t));
     }
   }
+  char* h = stage && stage->ensure(total) ? reinterpret_cast<char*>(stage->p) : nullptr;
+  for (int q = 0; q < np && e == cudaSuccess; q++)
+    e = cudaMemcpyAsync(h ? h + parts[q].off : parts[q].dst, parts[q].src, parts[q].bytes,
+                        cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_status(e);
+  for (int q = 0; q < np && h; q++) std::memcpy(parts[q].dst, h + parts[q].off, parts[q].bytes);
   if (herr & 1) return TRIOSEQ_ETIMEOUT;
   if (herr & 2) return TRIOSEQ_ECUDA;
   bt->have_rows = tb;
@@ -1487,7 +1504,7 @@ trioseq_status trioseq_align_batch(trioseq_plan_t plan, const trioseq_triplet* t
     s = run(bt.get(), st);
     plan->ws.mark_use(st);  // also after a partial enqueue: destroy waits for what did run
     if (s != TRIOSEQ_OK) return s;
-    if ((s = fetch(bt.get(), st, scores_out)) != TRIOSEQ_OK) return s;
+    if ((s = fetch(bt.get(), st, scores_out, &plan->ws.results)) != TRIOSEQ_OK) return s;
     bt->seq.clear();
     bt->seq.shrink_to_fit();
     plan->last = std::move(bt);
