@@ -41,7 +41,7 @@ size_t vl_smem(int KP) {
   const size_t prof = !CS ? (size_t)KP * (kPR * kPC * NJ / 2 + kPC * NH)
                           : (size_t)KP * (G::PJ16 + G::PK16) / 2;
   const size_t cv = CS ? (size_t)32 * 4 * G::CVG : 0;
-  return (sigN + (size_t)VlLaunch<NJ, NH, CS>::warps * (prof + kRing * G::SLOT + cv)) * sizeof(int);
+  return (sigN + (size_t)VlLaunch<NJ, NH, CS>::warps * (prof + kRing * G::SLOT + kVlRing + cv)) * sizeof(int);
 }
 }  // namespace
 

@@ -49,6 +49,8 @@ constexpr int kVlBias = 1 << 14;
 // -infinity reaches (8 + 3S + 7); with max sigma'' <= 30 that is [1216, 59904].
 constexpr int kVlTbBias = 11776;  // a multiple of 8
 
+constexpr int kVlRing = 64;  // slices in the residue ring
+
 template <int NJ, int NH>
 struct VlGeom {
   static constexpr int NK = 2 * NH;                  // cell columns per lane
@@ -69,13 +71,13 @@ struct VlGeom {
 // Two warps per sub-partition all but saturate it (32 x 64 tasks without waits: a step per 0.34 us with
 // one, 0.27 with two, 0.26 with three), and a third would need the 8 x 4 tile in 168 registers: protein 1,000
 // residues 0.67 -> 0.85 ms. The cap of 224 registers that `blocks` = 9 gives still leaves two; its code is the
-// faster (protein 4,000 residues 17.5 -> 17.2 ms, DNA traceback 3,000 residues 10.9 -> 10.1 ms), but not for
-// semi-global, where it spills (19.3 -> 19.9 ms).
-template <int NJ, int NH, int CS, int AT = kGlobal>
+// faster with traceback (DNA, 3,000 residues 11.3 -> 10.5 ms), the slower without (protein, 1,000 residues 0.649
+// -> 0.653 ms, semi-global, where it spills, 4.09 -> 4.27, local 1,500 1.80 -> 2.20).
+template <int NJ, int NH, int CS, int AT = kGlobal, bool TB = false>
 struct VlLaunch {
   static constexpr int warps = CS == 1 ? 2 : 1;
   static constexpr int blocks =
-      CS == 1 ? 5 : (CS == 2 ? 9 : (NH >= 8 ? 8 : (NJ >= 8 ? (AT == kSemiGlobal ? 8 : 9) : 12)));
+      CS == 1 ? 5 : (CS == 2 ? 9 : (NH >= 8 ? 8 : (NJ >= 8 ? (TB ? 9 : 8) : 12)));
   static constexpr int regs = 65536 / (warps * 32 * blocks) / 8 * 8;
   static constexpr int max_regs = regs > 255 ? 255 : regs;
 };
@@ -212,8 +214,8 @@ __device__ __forceinline__ void ld_halves(const unsigned short* p, unsigned (&v)
 // 103 (add-max with one), so operand reads bind a full sub-partition; the rest of a launch is the
 // chain of column tasks.
 template <int NJ, int NH, int CS, int AT, bool TB>
-__global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
-    __maxnreg__((VlLaunch<NJ, NH, CS, AT>::max_regs)) wavefront_vl_kernel(const WaveParams p) {
+__global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT, TB>::warps * 32)
+    __maxnreg__((VlLaunch<NJ, NH, CS, AT, TB>::max_regs)) wavefront_vl_kernel(const WaveParams p) {
   static_assert(AT == kGlobal || CS == 0, "the variant types keep sigma'' in registers");
   static_assert(!TB || (AT == kGlobal && CS == 0 && NH == 4), "traceback keys: global, NH = 4");
   using G = VlGeom<NJ, NH>;
@@ -223,6 +225,16 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
   constexpr int NEG = NEGH * 0x10001;   // in both halves
   constexpr int BIAS = TB ? kVlTbBias : kVlBias;
   constexpr int kOffJ = TB ? 3 : 0, kOffK = TB ? 2 : 0, kOffC = TB ? 1 : 0;  // rank offsets
+  // Two forms of a step, each where it is the faster (a step is bound by issue and by what the compiler lets
+  // its loads share a scoreboard with, so neither is everywhere):
+  // kXR: residues of S0 from a ring in shared memory instead of a global load per step. Local, protein 1,500
+  // residues 2.00 -> 1.80 ms; global, 4,000 residues 17.4 -> 17.9, 1,024 semi-global triplets 4.1 -> 5.0.
+  // kPK: right-column halves go to the next lane as the words the records hold, two rows each: half the
+  // shuffles and selects. Protein 4,000 residues 17.4 -> 17.25 ms, 1,000 0.665 -> 0.644; DNA traceback, 3,000
+  // residues 10.5 -> 11.9, local 1,500 2.00 -> 2.16.
+  constexpr bool kXR = AT == kLocal && NJ == 8 && NH == 4;
+  constexpr bool kPK = AT == kGlobal && !TB && CS == 0 && NJ == 8 && NH == 4;
+  constexpr int NCV = kPK ? NJ / 2 : NJ;  // column words a step takes from the left lane
   constexpr int W = NJ * NK / 8;        // TB: code words per lane per step
   extern __shared__ int4 smem4[];
   int* smem = reinterpret_cast<int*>(smem4);
@@ -242,13 +254,14 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
   constexpr bool kPT = !CS;
   const int prof_ints =
       kPT ? KP * (kPR * kPC * NJ / 2 + kPC * NH) : KP * (G::PJ16 + G::PK16) / 2;
-  const int warp_ints = prof_ints + kRing * G::SLOT + (CS ? 32 * 4 * G::CVG : 0);
+  const int warp_ints = prof_ints + kRing * G::SLOT + kVlRing + (CS ? 32 * 4 * G::CVG : 0);
   int* prof = smem + sigN + warp * warp_ints;
   unsigned short* profJ = reinterpret_cast<unsigned short*>(prof);
   unsigned short* profK =
       reinterpret_cast<unsigned short*>(prof + (kPT ? KP * kPR * kPC * NJ / 2 : KP * G::PJ16 / 2));
   int* ring = prof + prof_ints;
-  int4* cvs = reinterpret_cast<int4*>(ring + kRing * G::SLOT);  // CS only
+  int* xr = ring + kRing * G::SLOT;  // kXR: residues by slice
+  int4* cvs = reinterpret_cast<int4*>(xr + kVlRing);  // CS only
   // this lane's profile entries: J of residue x at pJ + x * kSJ, K at pKl / pKh + x * kSK
   constexpr int kSJ = kPT ? kPR * kPC * NJ : G::PJ16, kSK = kPT ? kPC * NH : G::PK16;
   const unsigned short* pJ = profJ + (kPT ? lane * NJ : r * NJ);
@@ -366,6 +379,9 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
     unsigned key_mask = 0xfff8fff8u, key_low = 0x00030003u;
     if (TB) asm volatile("" : "+r"(key_mask), "+r"(key_low));
     int P[NJ][NH];
+    int pk[NJ / 2];  // the right column's high halves, two rows a word
+#pragma unroll
+    for (int e = 0; e < NJ / 2; ++e) pk[e] = NEG;
     int rowA[NH + 1], colA[NJ], rowB[NH + 1], colB[NJ];
 #pragma unroll
     for (int pp = 0; pp < NJ; ++pp) {
@@ -537,7 +553,19 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
     }
     int xlast = xc;
     xc = xq;
-    xq = residue(s00 + 2);
+    // kXR: the residues from slice s + 2 on come from a ring of two blocks of 32 slices (block n covers slices
+    // 32n .. 32n + 31), a block being stored in the middle of the one before, when the block it replaces is
+    // behind every lane.
+    if constexpr (kXR) {
+      xr[lane] = residue(lane);
+      xr[32 + lane] = VIRT;  // the slices before 0
+      __syncwarp();
+    } else {
+      xq = residue(s00 + 2);
+    }
+    const auto refill = [&](const int t) {
+      if (kXR && (t & 31) == 16) xr[(t + 16 + lane) & (kVlRing - 1)] = residue(t + 16 + lane);
+    };
 
     // One step: the halo of slice s goes into rowCur / colCur, slice s - 1 is in rowPrev / colPrev.
     // inner: every lane has 1 <= s < a, so no lane needs a range check, a reset or end-cell work,
@@ -562,7 +590,8 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
       for (int q4 = 0; q4 < NH / 4; ++q4)
         st_ring_row(st_w + o + 16 * q4, w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3], f_j);
       st_ring_corner(st_c + o, cw, f_j);
-      st_ring_col<NJ>(st_w + o, w, f_k);
+      if constexpr (kPK) st_ring_row(st_w + o, w[0], w[1], w[2], w[3], f_k);
+      else st_ring_col<NJ>(st_w + o, w, f_k);
       if (inner || t + 2 < T) fetch(t + 2, inner);
       __syncwarp();
       return true;
@@ -587,19 +616,22 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
       ld_halves<NH>(pKl + xc * kSK, kl);
       ld_halves<NH>(pKh + xlast * kSK, kh);
       xlast = xc;
-      xc = xq;
-      xq = inner ? (int)__ldg(S0 + (s + 2)) : residue(s + 3);
+      if constexpr (kXR) {
+        xc = xr[(s + 2) & (kVlRing - 1)];
+      } else {
+        xc = xq;
+        xq = inner ? (int)__ldg(S0 + (s + 2)) : residue(s + 3);
+      }
       // Halo of slice s from the neighbour lanes' previous step; the edge lanes take the staged
-      // words instead. Column words: this row's value in the high half.
+      // words instead. Column words: this row's value in the high half (kPK: two rows' values).
 #pragma unroll
       for (int qq = 0; qq <= NH; ++qq)
         rowCur[qq] = __shfl_up_sync(kFull, qq == 0 ? colPrev[NJ - 1] : P[NJ - 1][qq - 1], kPC);
-      int cv_[NJ], mine[NJ];
+      int cv_[NCV], mine[NJ];
 #pragma unroll
-      for (int pp = 0; pp < NJ; ++pp) {
-        mine[pp] = P[pp][NH - 1];
-        cv_[pp] = __shfl_up_sync(kFull, mine[pp], 1);
-      }
+      for (int pp = 0; pp < NJ; ++pp) mine[pp] = P[pp][NH - 1];
+#pragma unroll
+      for (int w = 0; w < NCV; ++w) cv_[w] = __shfl_up_sync(kFull, kPK ? pk[w % (NJ / 2)] : mine[w], 1);
       {
         const int* q = ring + slot * G::SLOT;
         const int corner = q[G::RC + lc];
@@ -613,7 +645,7 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
           rowCur[4 + 4 * q4] = r == 0 ? w.w : rowCur[4 + 4 * q4];
         }
 #pragma unroll
-        for (int p4 = 0; p4 < NJ / 4; ++p4) {
+        for (int p4 = 0; p4 < NCV / 4; ++p4) {
           const int4 w = reinterpret_cast<const int4*>(q + G::RQ + r * NJ)[p4];
           cv_[4 * p4] = lc == 0 ? w.x : cv_[4 * p4];
           cv_[4 * p4 + 1] = lc == 0 ? w.y : cv_[4 * p4 + 1];
@@ -623,7 +655,8 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
       }
 #pragma unroll
       for (int pp = 0; pp < NJ; ++pp)
-        colCur[pp] = (int)__byte_perm((unsigned)cv_[pp], (unsigned)mine[pp], 0x5432);
+        colCur[pp] = (int)__byte_perm((unsigned)cv_[kPK ? pp / 2 : pp], (unsigned)mine[pp],
+                                      kPK && pp % 2 == 0 ? 0x5410 : 0x5432);
       // Axis feeds. Only two kinds of halo cells are finite: those of slice -1 (each lane meets slice -1
       // once, the step before its first) and the i-axis feed M'[s][-1][-1] of lane 0 of task (0, 0);
       // every other halo cell of the first row or column stays -infinity, as staged.
@@ -770,12 +803,11 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
         }
         {
           int* q = dstK + (int64_t)t * G::RK;
-          int w[4] = {0, 0, 0, 0};
 #pragma unroll
           for (int e = 0; e < NJ / 2; ++e)
-            w[e] = (int)__byte_perm((unsigned)P[2 * e][NH - 1], (unsigned)P[2 * e + 1][NH - 1],
-                                    0x7632);
-          vl_store(q, w[0], w[1], w[2], w[3], q + kPR * 4 - r * 2, Bt, Bt,
+            pk[e] = (int)__byte_perm((unsigned)P[2 * e][NH - 1], (unsigned)P[2 * e + 1][NH - 1],
+                                     0x7632);
+          vl_store(q, pk[0], pk[1], NJ == 8 ? pk[NJ / 2 - 2] : 0, NJ == 8 ? pk[NJ / 2 - 1] : 0, q + kPR * 4 - r * 2, Bt, Bt,
                    inner ? f_ok : (s >= 1 ? f_ok : 0));
         }
         const int ub = Bt - BIAS;  // biased half -> absolute M' (or key)
@@ -870,6 +902,10 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
             P[pp][qq] = (int)(__vmaxu2((unsigned)P[pp][qq], mn) - m);
           colB[pp] = (int)(__vmaxu2((unsigned)colB[pp], mn) - m);
         }
+        if constexpr (kPK) {
+#pragma unroll
+          for (int e = 0; e < NJ / 2; ++e) pk[e] = (int)(__vmaxu2((unsigned)pk[e], mn) - m);
+        }
 #pragma unroll
         for (int qq = 0; qq <= NH; ++qq) rowB[qq] = (int)(__vmaxu2((unsigned)rowB[qq], mn) - m);
         Bt += dlt;
@@ -884,6 +920,7 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT>::warps * 32)
     // different phases: the 300-residue protein triplet 0.19 -> 0.23 ms, 1,024 triplets 3.7 -> 4.6 ms.
     auto pair = [&](const int t, const bool inner) -> bool {
       const int slot = t & 2;
+      refill(t);
       if (!stage(t, inner, slot)) return false;
       step(t, inner, slot, jA, jB, rowA, rowB, colA, colB);
       if (inner || t + 1 < T) step(t + 1, inner, slot + 1, jB, jA, rowB, rowA, colB, colA);
