@@ -136,7 +136,7 @@ struct Workspace {
   DevBuf walkstate; // slab mode: (i, j, k, n) of the traceback walk between slabs
   DevBuf best64;    // semi-global / local traceback: (score, first cell) key per triplet
   DevBuf spans;     // traceback: begin and end cell of each alignment (6 int32)
-  HostPinned staging, results;  // per-call path: inputs up, results down
+  HostPinned staging;  // per-call path: inputs up, then room for the results down
   // Buffers are allocated and freed in this stream's order. Plans and device-resident batches
   // own a private stream here (own_stream); a serving slot uses its launch stream.
   cudaStream_t alloc_stream = nullptr;
@@ -918,6 +918,13 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
 }
 
 
+// Bytes of a run's results as fetch() stages them: error word, scores, rows, lengths and spans.
+size_t results_bytes(const trioseq_batch_s* bt) {
+  const size_t ntb = bt->tb_trips.size();
+  return 64 + align_up(bt->n * 4, 64) +
+         (ntb ? align_up(bt->rows_bytes, 64) + align_up(ntb * 4, 64) + align_up(ntb * 24, 64) : 0);
+}
+
 // Size the workspace and copy the inputs of `bt` into it (stream-ordered).
 // `pinned`: stage through the workspace's pinned buffer and copy asynchronously on `st` (the
 // per-call path); otherwise copy synchronously from pageable memory (one-off batch creation).
@@ -940,7 +947,7 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
                               as)) ||
       (tb && plan_atype(bt) != kGlobal &&
        !ws.best64.ensure(std::max<size_t>(bt->n, 1) * sizeof(unsigned long long), as)) ||
-      (pinned && !ws.staging.ensure(bt->inputs_bytes)))
+      (pinned && !ws.staging.ensure(align_up(bt->inputs_bytes, 256) + results_bytes(bt))))
     return TRIOSEQ_ENOMEM;
   // On a private allocation stream, the buffers are ready before any launch stream uses them.
   if (ws.own_stream && cudaStreamSynchronize(as) != cudaSuccess)
@@ -1226,12 +1233,13 @@ trioseq_status run_graph(trioseq_batch_s* bt, cudaStream_t st) {
   return TRIOSEQ_OK;
 }
 
-// Wait for the run, check the error word, fetch scores (and traceback rows). With `stage`, the copies go to
-// that pinned buffer, enqueued behind the run, and are handed on after one wait (a copy to pageable memory
-// holds the caller for its own round trip: 48 us for the five of a call with rows, 22 us for the two of a score
-// call, against 9 and 6); without, straight to their destinations, which several threads may do at once.
+// Wait for the run, check the error word, fetch scores (and traceback rows). `staged` (after an upload through
+// the pinned buffer): the copies go to that buffer, behind the inputs and enqueued behind the run, and are
+// handed on after one wait (a copy to pageable memory holds the caller for its own round trip: 48 us for the
+// five of a call with rows, 22 us for the two of a score call, against 16 and 12). Without, straight to their
+// destinations, which several threads may do at once.
 trioseq_status fetch(trioseq_batch_s* bt, cudaStream_t st, int32_t* scores_out,
-                     HostPinned* stage = nullptr) {
+                     bool staged = false) {
   Workspace& ws = *bt->ws;
   const bool tb = bt->mode == TRIOSEQ_WITH_TRACEBACK;
   int32_t herr = 0;
@@ -1260,7 +1268,9 @@ trioseq_status fetch(trioseq_batch_s* bt, cudaStream_t st, int32_t* scores_out,
       add(bt->h_spans.data(), ws.spans.p, bt->h_spans.size() * sizeof(int32_t));
     }
   }
-  char* h = stage && stage->ensure(total) ? reinterpret_cast<char*>(stage->p) : nullptr;
+  const size_t at = align_up(bt->inputs_bytes, 256);
+  char* h = staged && at + total <= ws.staging.cap ? reinterpret_cast<char*>(ws.staging.p) + at
+                                                   : nullptr;
   for (int q = 0; q < np && e == cudaSuccess; q++)
     e = cudaMemcpyAsync(h ? h + parts[q].off : parts[q].dst, parts[q].src, parts[q].bytes,
                         cudaMemcpyDeviceToHost, st);
@@ -1504,7 +1514,7 @@ trioseq_status trioseq_align_batch(trioseq_plan_t plan, const trioseq_triplet* t
     s = run(bt.get(), st);
     plan->ws.mark_use(st);  // also after a partial enqueue: destroy waits for what did run
     if (s != TRIOSEQ_OK) return s;
-    if ((s = fetch(bt.get(), st, scores_out, &plan->ws.results)) != TRIOSEQ_OK) return s;
+    if ((s = fetch(bt.get(), st, scores_out, true)) != TRIOSEQ_OK) return s;
     bt->seq.clear();
     bt->seq.shrink_to_fit();
     plan->last = std::move(bt);
