@@ -563,8 +563,9 @@ Variant default_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip,
 // most two tasks per SM). Kernel time, 8x4 / 4x8 / 4x4 / 8x8: 4,096 DNA triplets of 100..300 residues
 // 11.2 / 11.8 / 12.2 / 13.3 ms, of 30..60 260 / 243 / 243 / 350 us; 100 of 60..100 77 / 78 / 82 / 129 us; 8 of
 // 100..200 132 / 138 / 115 / 223 us; 300 protein triplets of 100..200 436 / 460 / 440 / 571 us.
+// 8x8 (32 x 64), whose records are two thirds of 8x4's, where those would exceed the plan's record budget.
 Variant packed_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n) {
-  double tasks = 0, wide = 0, narrow = 0;  // tasks of 8x4; padded cells of 8x4 and 4x4
+  double tasks = 0, wide = 0, narrow = 0;  // tasks of 8x4; steps of 8x4 and 4x4 tasks, in 16 x 32 blocks
   for (size_t t = 0; t < n; t++) {
     const double a = trip[t].len[0] + 11.0, k = (trip[t].len[2] + 32) / 32;
     const double j8 = (trip[t].len[1] + 32) / 32, j4 = (trip[t].len[1] + 16) / 16;
@@ -572,7 +573,11 @@ Variant packed_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip, 
     wide += a * j8 * k * 2;
     narrow += a * j4 * k;
   }
-  return tasks <= 2.0 * plan->sms || 1.08 * narrow < wide ? Variant{4, 4} : Variant{8, 4};
+  const bool few = tasks <= 2.0 * plan->sms || 1.08 * narrow < wide;
+  const double bytes = few ? 0.5 * narrow * 4 * (vp_rec_j(4) + vp_rec_k(4))
+                           : 0.25 * wide * 4 * (vp_rec_j(4) + vp_rec_k(8));
+  if (bytes > (double)plan->slab_budget) return Variant{8, 8};
+  return few ? Variant{4, 4} : Variant{8, 4};
 }
 
 // Build the host side of a batch: encode, pack, describe, order the queue.

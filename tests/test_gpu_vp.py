@@ -29,8 +29,8 @@ def _plan(sc, **env):
                 os.environ[k] = v
 
 
-def _check(sc, trips, tile=None):
-    plan = _plan(sc, **({"TRIOSEQ_SCORE_TILE": tile} if tile else {}))
+def _check(sc, trips, tile=None, **env):
+    plan = _plan(sc, **({"TRIOSEQ_SCORE_TILE": tile} if tile else {}), **env)
     try:
         bt = B.trioseq_batch_create(plan, [[synth.to_str(s, sc.alphabet) for s in t] for t in trips])
         try:
@@ -81,3 +81,8 @@ def test_alphabets(tile, K):
 def test_tile_rule(n, lo, hi, tile):
     w = synth.config2(seed=704, n=n, lo=lo, hi=hi)
     assert _check(DNA, w.triplets) == tile
+
+
+def test_tile_rule_over_the_record_budget():
+    w = synth.config2(seed=705, n=40, lo=100, hi=200)
+    assert _check(DNA, w.triplets, TRIOSEQ_SLAB_BUDGET_MB=1) == (8, 8)
