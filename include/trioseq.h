@@ -266,9 +266,10 @@ trioseq_status trioseq_batch_timing(trioseq_batch_t batch, float ms[2]);
  * fastest in the plan for batches of the same mode, the same single-or-batch kind, and the same
  * bit length of the longest sequence. Later batches of that class use it; other classes keep
  * the defaults: where the scheme admits two cells per register, tile 4x8v for batches of at most
- * two 16x64 column tasks per SM and 8x8v beyond; int32 (8x8 score-only, 4x8 traceback, interval 8)
- * elsewhere, and for some global batches of at most 8 such tasks or of two triplets of which one is a
- * single task; global score batches whose pairs fit 16-bit halves run two triplets per register. Outputs (any may be null) report
+ * two 16x64 column tasks per SM and 8x8v beyond; int32 elsewhere (8x8 score-only, 4x8 traceback, 4x4
+ * semi-global and local traceback, interval 8), and for some global batches of at most 8 such tasks or of
+ * two triplets of which one is a single task; global score batches whose pairs fit 16-bit halves run two
+ * triplets per register. Outputs (any may be null) report
  * the choice. The plan's device memory is untouched; a temporary workspace is used.
  * Errors: EINVAL, EOVERFLOW, ENOMEM, ETIMEOUT, ECUDA. */
 trioseq_status trioseq_plan_autotune(trioseq_plan_t plan, const trioseq_triplet* sample, size_t n,

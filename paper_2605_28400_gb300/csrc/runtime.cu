@@ -580,6 +580,19 @@ Variant packed_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip, 
   return few ? Variant{4, 4} : Variant{8, 4};
 }
 
+// The int32 tile of a semi-global or local batch with traceback: 4x4 (16 x 32 tasks), whose one-pass step with
+// its best-cell bookkeeping keeps to fewer registers, unless its records (0.41 B a cell against 0.33 on 4x8)
+// and the codes exceed the plan's budget. Kernel time, 4x8 / 8x4 / 4x4: local, DNA, 100 residues 375 / 330 / 238 us,
+// 1,000 4.0 / 3.9 / 3.2 ms, protein, 1,700 13.9 / 14.1 / 10.5; semi-global, DNA, 1,000 3.2 / 3.0 / 2.4 ms, protein,
+// 1,700 8.8 / 8.7 / 7.4; 60 DNA triplets of 100..400 local 4.0 / 3.9 / 2.9, semi-global 3.3 / 3.0 / 2.2.
+Variant typed_tb_tile(const trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n) {
+  double bytes = 0;
+  for (size_t t = 0; t < n; t++)
+    bytes += (trip[t].len[0] + 11.0) * ((trip[t].len[1] + 16) / 16) * ((trip[t].len[2] + 32) / 32) *
+             (4.0 * (kPC * 4 + 4 + kPR * 4) + 32.0 * 2 * 4);
+  return bytes <= (double)plan->slab_budget ? Variant{4, 4} : Variant{4, 8};
+}
+
 // Build the host side of a batch: encode, pack, describe, order the queue.
 trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n,
                            uint32_t mode, trioseq_batch_s* bt) {
@@ -640,7 +653,8 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
     }
     if (!ok_vl) {
       if (plan->tuning) return TRIOSEQ_ECUDA;  // the autotuner skips the candidate
-      bt->var = tb ? Variant{4, 8} : Variant{8, 8};  // the int32 defaults
+      // the int32 defaults
+      bt->var = tb ? (plan->atype != kGlobal ? typed_tb_tile(plan, trip, n) : Variant{4, 8}) : Variant{8, 8};
     }
   }
   const int NJ = bt->var.nj, NK = bt->var.nk;
@@ -910,7 +924,9 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   int bpm = 0;
   // Int32 traceback launches of one triplet use the records as readiness flags; TRIOSEQ_DATA_FLAGS at
   // plan creation forces it on (1) or off (0). (The two-cells-per-register kernel always does.)
-  bt->df = tb && !vl && !bt->slab && (plan->data_flags >= 0 ? plan->data_flags != 0 : n == 1);
+  // Batches of the semi-global and local types too: 60 DNA triplets of 100..400 2.9 -> 2.5 and 2.2 -> 1.9 ms.
+  bt->df = tb && !vl && !bt->slab &&
+           (plan->data_flags >= 0 ? plan->data_flags != 0 : n == 1 || plan->atype != kGlobal);
   if (wavefront_occupancy(NJ, NK, tb, plan->atype, bt->packed, bt->slab > 0, bt->smem,
                           &bpm) != 0 ||
       bpm <= 0)
@@ -1849,7 +1865,8 @@ struct SrvSlot {
 // traceback mode the code stream and rows).
 size_t request_bytes(const trioseq_plan_s* plan, uint32_t mode, const uint32_t len[3]) {
   const bool tb = mode == TRIOSEQ_WITH_TRACEBACK;
-  const Variant v = tb ? plan->tb_variant : plan->score_variant;
+  Variant v = tb ? plan->tb_variant : plan->score_variant;
+  if (auto_tile(plan, tb) && tb && plan->atype != kGlobal) v = Variant{4, 4};  // typed_tb_tile's larger one
   const size_t WJ = (size_t)kPR * v.nj, WK = (size_t)kPC * v.nk, W = (size_t)v.nj * v.nk / 8;
   const size_t a = len[0], b = len[1], c = len[2];
   const size_t nJ = (b + 1 + WJ - 1) / WJ, nK = (c + 1 + WK - 1) / WK, T = a + 1 + 10;

@@ -74,7 +74,7 @@ def test_narrow_tile_exact(sc, kind):
     ("local", B.SCORE_ONLY, [(30, 64, 127)], "4x8v"),
     ("semiglobal", B.SCORE_ONLY, [(9, 100, 100)] * 21, "4x8v"),        # 21 x 14 = 294 tasks
     ("semiglobal", B.SCORE_ONLY, [(9, 100, 100)] * 22, "8x8v"),        # 308: past two per SM (152)
-    ("local", B.WITH_TRACEBACK, [(30, 64, 127)], "4x8"),               # no such keys: int32
+    ("local", B.WITH_TRACEBACK, [(30, 64, 127)], "4x4"),               # no such keys: int32
     ("global", B.SCORE_ONLY, [(30, 64, 127), (20, 30, 40)], "4x4"),    # packs two triplets
 ], ids=str)
 def test_default_tile(kind, mode, shapes, label):
