@@ -185,7 +185,7 @@ def _triplet_array(triplets):
     if n and set(map(len, triplets)) != {3}:
         raise ValueError("a triplet has three sequences")
     if n == 1:  # one record, without the arrays below
-        parts = triplets[0]
+        parts = next(iter(triplets))  # any sized collection, as above: no index
         if all(isinstance(x, str) for x in parts):
             parts = [x.encode("latin-1") for x in parts]
         else:
