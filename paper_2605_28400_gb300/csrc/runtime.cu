@@ -585,7 +585,14 @@ Variant packed_variant(const trioseq_plan_s* plan, const trioseq_triplet* trip, 
 // and the codes exceed the plan's budget. Kernel time, 4x8 / 8x4 / 4x4: local, DNA, 100 residues 375 / 330 / 238 us,
 // 1,000 4.0 / 3.9 / 3.2 ms, protein, 1,700 13.9 / 14.1 / 10.5; semi-global, DNA, 1,000 3.2 / 3.0 / 2.4 ms, protein,
 // 1,700 8.8 / 8.7 / 7.4; 60 DNA triplets of 100..400 local 4.0 / 3.9 / 2.9, semi-global 3.3 / 3.0 / 2.2.
+// One triplet whose third sequence is by far the longest is a chain of column tasks along k, which 16 x 64 tasks
+// halve: c >= 12 a and c >= 4 b. Semi-global, 4x8 / 4x4, us: 20 x 20 x 3,000 803 / 978, 20 x 600 x 3,000
+// 1,047 / 1,156, 60 x 60 x 700 324 / 338; past the line 100 x 100 x 1,000 524 / 518, 300 x 300 x 2,500
+// 1,449 / 1,389, 20 x 500 x 500 353 / 311.
 Variant typed_tb_tile(const trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n) {
+  if (n == 1 && trip[0].len[2] >= 12.0 * std::max(1u, trip[0].len[0]) &&
+      trip[0].len[2] >= 4.0 * trip[0].len[1])
+    return Variant{4, 8};
   double bytes = 0;
   for (size_t t = 0; t < n; t++)
     bytes += (trip[t].len[0] + 11.0) * ((trip[t].len[1] + 16) / 16) * ((trip[t].len[2] + 32) / 32) *
