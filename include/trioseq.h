@@ -125,8 +125,11 @@ trioseq_status trioseq_plan(const trioseq_scoring* scoring, uint32_t max_len_hin
  * TRIOSEQ_GLOBAL. The plan serves trioseq_align_batch and the device-resident batch calls in
  * score-only mode (traceback: ENOTIMPL); trioseq_plan_autotune has nothing to choose. The
  * kernel keeps 13 values per cell in the linear engine's column tasks, two triplets per register
- * when a batch's values fit 16 bits; a triplet whose boundary records (2.5 bytes per cell of the
- * cube, 1.25 packed) exceed the plan's budget (trioseq_batch_slabs) sweeps anti-diagonal planes.
+ * when a batch's values fit 16 bits; large batches run as launches over the same 4 GB of boundary
+ * records. A triplet whose records (2.5 bytes per cell of the cube, 1.25 packed) exceed the plan's
+ * budget (trioseq_batch_slabs), or for which the device has no room, makes its batch sweep
+ * anti-diagonal planes instead (256 bytes per cell of a (j, k) plane, several hundred times
+ * slower). Between calls a plan keeps at most 16 GB of records.
  * Errors: EINVAL (as trioseq_plan, gap_open out of range, other flags), ENOMEM, ECUDA;
  * EOVERFLOW at batch time when (3 max|sub| + 3|gap| + 3|gap_open|) * (a+b+c) >= 2^29. */
 trioseq_status trioseq_plan_affine(const trioseq_scoring* scoring, int32_t gap_open,
@@ -146,7 +149,8 @@ trioseq_status trioseq_plan_destroy(trioseq_plan_t plan);
  * trioseq_traceback.
  * Work: encode + pack (host), one H2D copy, one persistent wavefront launch over all triplets,
  * one traceback-walk launch (traceback mode), one D2H copy of scores (and alignments).
- * Errors: EINVAL (residue outside the alphabet, null), EOVERFLOW, ENOMEM, ETIMEOUT, ECUDA. */
+ * Errors: EINVAL (residue outside the alphabet, null), EOVERFLOW, ENOMEM (after smaller layouts of
+ * the records and codes, where there are any, found no room either), ETIMEOUT, ECUDA. */
 trioseq_status trioseq_align_batch(trioseq_plan_t plan, const trioseq_triplet* triplets, size_t n,
                                    uint32_t mode, int32_t* scores_out, void* stream);
 

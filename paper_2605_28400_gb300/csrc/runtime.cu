@@ -283,6 +283,7 @@ struct trioseq_batch_s {
   size_t plane_ints = 0, nplanes = 0, off_slab = 0;
   std::vector<TripDesc> slab_desc;
   bool uploaded = false;
+  bool no_room = false;  // the last upload failed for its boundary records or codes
   // results of the last run (host)
   std::vector<uint8_t> h_rows;
   std::vector<int32_t> h_lens;
@@ -382,12 +383,16 @@ trioseq_status build_affine_planes(trioseq_plan_s* plan, trioseq_batch_s* bt) {
 // cube first). The boundary records take 2.5 bytes per cell of the grid, so large batches run as
 // chunks, one launch after another over the same records: 4 GB hold about ten waves of tasks of
 // 200-residue triplets, so the tail of a chunk costs little. A triplet whose records exceed the
-// plan's budget runs over planes instead (64 bytes per cell of a (j, k) plane).
-trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt) {
+// plan's budget runs over planes instead (four planes of 64 bytes per (j, k) cell).
+// lean: the layout to build when the device had no room for a larger one: 1 the smallest chunks, 2 planes.
+constexpr size_t kAffineChunkInts = (size_t)1 << 30;  // 4 GB
+constexpr size_t kAffineKeep = (size_t)16 << 30;      // bytes of records a plan keeps between calls
+trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt, int lean) {
   const size_t n = bt->n;
   bt->seq_bytes = bt->seq.size();
   bt->affine_chunks.clear();
   bt->affine_cells = 0;
+  if (lean >= 2) return build_affine_planes(plan, bt);
   const auto volume = [&](int32_t t) {
     const TripDesc& d = bt->desc[t];
     return (double)(d.len[0] + 1) * (d.len[1] + 1) * (d.len[2] + 1);
@@ -440,7 +445,7 @@ trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt) {
     return (size_t)d.nJ * d.nK * (size_t)(d.glen[0] + 1) * (size_t)(kAffineRecJ + kAffineRecK);
   };
   const size_t budget = plan->slab_budget / 4;
-  size_t limit = std::min(budget, (size_t)1 << 30);  // ints
+  size_t limit = lean ? 0 : std::min(budget, kAffineChunkInts);
   for (const auto& un : units) {
     const size_t rec = records(bt->desc[un.first]);
     if (rec > budget) {
@@ -600,9 +605,11 @@ Variant typed_tb_tile(const trioseq_plan_s* plan, const trioseq_triplet* trip, s
   return bytes <= (double)plan->slab_budget ? Variant{4, 4} : Variant{4, 8};
 }
 
-// Build the host side of a batch: encode, pack, describe, order the queue.
+// Build the host side of a batch: encode, pack, describe, order the queue. lean > 0: a layout for a device
+// that had no room for the batch's first one (make_batch): int32 tiles, or pairs on their 8x8 tile; affine
+// gaps as build_affine says.
 trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n,
-                           uint32_t mode, trioseq_batch_s* bt) {
+                           uint32_t mode, trioseq_batch_s* bt, int lean = 0) {
   if (!trip && n) return TRIOSEQ_EINVAL;
   if (mode > TRIOSEQ_WITH_TRACEBACK) return TRIOSEQ_EINVAL;
   const bool tb = mode == TRIOSEQ_WITH_TRACEBACK;
@@ -619,6 +626,8 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
     if (plan->tuning) {
       bt->var = plan->forced.var;
       bt->TI = plan->forced.TI;
+    } else if (lean) {
+      if (!(tb ? plan->tb_forced : plan->score_forced)) bt->var = tb ? Variant{4, 8} : Variant{8, 8};
     } else {
       auto it = plan->tuned.find(tune_key(mode, n, maxlen));
       if (it != plan->tuned.end()) {
@@ -765,7 +774,7 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   }
   if (plan->affine) {
     if (tb) return TRIOSEQ_ENOTIMPL;  // the affine model is score-only on the device
-    return build_affine(plan, bt);
+    return build_affine(plan, bt, lean);
   }
   // 2. Units of work: one triplet, or in packed int16x2 mode two triplets of the same column-task
   //    grid class paired in one unit (the high halves run on the grid of their maximal lengths).
@@ -963,11 +972,9 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
   cudaStream_t as = ws.alloc_stream;
   ws.order_after_last_use();  // a buffer that grows is freed only after its last use
   if (!ws.inputs.ensure(bt->inputs_bytes, as) ||
-      !ws.faces.ensure(bt->face_ints * sizeof(int32_t), as) ||
       !ws.progress.ensure(nprog * sizeof(int32_t), as) ||
       !ws.scores.ensure(std::max<size_t>(bt->n, 1) * sizeof(int32_t), as) ||
-      (tb && (!ws.codes.ensure(bt->code_words * sizeof(uint32_t), as) ||
-              !ws.rows.ensure(bt->rows_bytes, as) ||
+      (tb && (!ws.rows.ensure(bt->rows_bytes, as) ||
               !ws.lens.ensure(std::max<size_t>(bt->tb_trips.size(), 1) * sizeof(int32_t), as))) ||
       (bt->nplanes && !ws.planes.ensure(bt->nplanes * bt->plane_ints * sizeof(int32_t), as)) ||
       (bt->slab && tb && !ws.walkstate.ensure(4 * sizeof(int32_t), as)) ||
@@ -977,6 +984,10 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
        !ws.best64.ensure(std::max<size_t>(bt->n, 1) * sizeof(unsigned long long), as)) ||
       (pinned && !ws.staging.ensure(align_up(bt->inputs_bytes, 256) + results_bytes(bt))))
     return TRIOSEQ_ENOMEM;
+  // the records and codes last: their size is the layout's choice (make_batch)
+  bt->no_room = !ws.faces.ensure(bt->face_ints * sizeof(int32_t), as) ||
+                (tb && !ws.codes.ensure(bt->code_words * sizeof(uint32_t), as));
+  if (bt->no_room) return TRIOSEQ_ENOMEM;
   // On a private allocation stream, the buffers are ready before any launch stream uses them.
   if (ws.own_stream && cudaStreamSynchronize(as) != cudaSuccess)
     return cuda_status(cudaGetLastError());
@@ -1009,6 +1020,39 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
   bt->uploaded = true;
   bt->h2d_bytes = bt->inputs_bytes;
   return TRIOSEQ_OK;
+}
+
+// Build a batch and place it in `ws` (or a workspace of its own). Where the device has no room for the records
+// and codes of the default layout, the layouts that need less are tried before the call fails.
+trioseq_status make_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n, uint32_t mode,
+                          Workspace* ws, cudaStream_t st, bool pinned,
+                          std::unique_ptr<trioseq_batch_s>* out) {
+  size_t refused = SIZE_MAX;  // bytes of the layout that found no room
+  trioseq_status s = TRIOSEQ_ENOMEM;
+  for (int lean = 0; lean <= (plan->affine ? 2 : 1); lean++) {
+    std::unique_ptr<trioseq_batch_s> bt(new (std::nothrow) trioseq_batch_s());
+    if (!bt) return TRIOSEQ_ENOMEM;
+    if (const trioseq_status b = build_batch(plan, trip, n, mode, bt.get(), lean); b != TRIOSEQ_OK)
+      return b;
+    const size_t bytes = 4 * (bt->face_ints + (mode == TRIOSEQ_WITH_TRACEBACK ? bt->code_words : 0) +
+                              bt->nplanes * bt->plane_ints);
+    if (bytes >= refused) continue;
+    if (!ws) {
+      bt->own_ws.reset(new (std::nothrow) Workspace());
+      if (!bt->own_ws) return TRIOSEQ_ENOMEM;
+      if (bt->own_ws->make_own_stream() != cudaSuccess) return cuda_status(cudaGetLastError());
+    }
+    bt->ws = ws ? ws : bt->own_ws.get();
+    s = upload(bt.get(), st, pinned);
+    if (s == TRIOSEQ_OK) *out = std::move(bt);
+    if (s == TRIOSEQ_OK || !bt->no_room) return s;
+    refused = bytes;
+    if (ws) {  // what the larger layout did get
+      ws->faces.reset();
+      ws->codes.reset();
+    }
+  }
+  return s;
 }
 
 // Event record that also works inside a stream capture (there it becomes an event-record node
@@ -1532,17 +1576,22 @@ trioseq_status trioseq_align_batch(trioseq_plan_t plan, const trioseq_triplet* t
     if (!plan || (n && !scores_out)) return TRIOSEQ_EINVAL;
     DeviceGuard g(plan->device);
     cudaStream_t st = (cudaStream_t)stream;
-    std::unique_ptr<trioseq_batch_s> bt(new (std::nothrow) trioseq_batch_s());
-    if (!bt) return TRIOSEQ_ENOMEM;
+    std::unique_ptr<trioseq_batch_s> bt;
     plan->last.reset();
-    trioseq_status s = build_batch(plan, triplets, n, mode, bt.get());
+    trioseq_status s = make_batch(plan, triplets, n, mode, &plan->ws, st, true, &bt);
     if (s != TRIOSEQ_OK) return s;
-    bt->ws = &plan->ws;
-    if ((s = upload(bt.get(), st, true)) != TRIOSEQ_OK) return s;
     s = run(bt.get(), st);
     plan->ws.mark_use(st);  // also after a partial enqueue: destroy waits for what did run
     if (s != TRIOSEQ_OK) return s;
     if ((s = fetch(bt.get(), st, scores_out, true)) != TRIOSEQ_OK) return s;
+    // A plan keeps at most 16 GB of affine records from one call to the next: those of a triplet of 1,850
+    // residues. Beyond, they go back to the device and are taken again by the next call, which costs about as
+    // long as its kernel (2,000 residues, 20 GB: 35 -> 79 ms).
+    if (plan->affine && plan->ws.faces.cap > kAffineKeep) {
+      plan->ws.order_after_last_use();
+      plan->ws.faces.reset();
+      cudaStreamSynchronize(plan->ws.alloc_stream);  // the pool returns it at the next synchronisation
+    }
     bt->seq.clear();
     bt->seq.shrink_to_fit();
     plan->last = std::move(bt);
@@ -1574,15 +1623,9 @@ trioseq_status trioseq_batch_create(trioseq_plan_t plan, const trioseq_triplet* 
     if (!plan || !out) return TRIOSEQ_EINVAL;
     *out = nullptr;
     DeviceGuard g(plan->device);
-    std::unique_ptr<trioseq_batch_s> bt(new (std::nothrow) trioseq_batch_s());
-    if (!bt) return TRIOSEQ_ENOMEM;
-    trioseq_status s = build_batch(plan, triplets, n, mode, bt.get());
+    std::unique_ptr<trioseq_batch_s> bt;
+    const trioseq_status s = make_batch(plan, triplets, n, mode, nullptr, nullptr, false, &bt);
     if (s != TRIOSEQ_OK) return s;
-    bt->own_ws.reset(new (std::nothrow) Workspace());
-    if (!bt->own_ws) return TRIOSEQ_ENOMEM;
-    if (bt->own_ws->make_own_stream() != cudaSuccess) return cuda_status(cudaGetLastError());
-    bt->ws = bt->own_ws.get();
-    if ((s = upload(bt.get(), nullptr, false)) != TRIOSEQ_OK) return s;
     *out = bt.release();
     return TRIOSEQ_OK;
   });
@@ -1946,13 +1989,10 @@ trioseq_status srv_launch(trioseq_server_s* S, SrvSlot& sl) {
       trips[i].s[q] = sl.reqs[i].s[q].data();
       trips[i].len[q] = (uint32_t)sl.reqs[i].s[q].size();
     }
-  sl.batch.reset(new (std::nothrow) trioseq_batch_s());
-  if (!sl.batch) return TRIOSEQ_ENOMEM;
-  trioseq_batch_s* bt = sl.batch.get();
-  trioseq_status st = build_batch(plan, trips.data(), trips.size(), mode, bt);
+  trioseq_status st =
+      make_batch(plan, trips.data(), trips.size(), mode, &sl.ws, sl.stream, true, &sl.batch);
   if (st != TRIOSEQ_OK) return st;
-  bt->ws = &sl.ws;
-  if ((st = upload(bt, sl.stream, true)) != TRIOSEQ_OK) return st;
+  trioseq_batch_s* bt = sl.batch.get();
   NvtxRange range("trioseq_server_launch");
   if ((st = run(bt, sl.stream)) != TRIOSEQ_OK) return st;
   const bool tb = mode == TRIOSEQ_WITH_TRACEBACK;
