@@ -295,7 +295,8 @@ typedef struct trioseq_server_s* trioseq_server_t;
  * `hbm_budget` bytes (0 = 80% of the memory free at creation, and then each admission is also
  * bounded by the memory free on the device at that moment). One launch groups same-scheme,
  * same-mode requests up to a quarter of the budget; a single larger request (up to the whole
- * budget; a global-type triplet counted at its slab workspace, see trioseq_batch_slabs) waits in
+ * budget; a global-type triplet counted at its slab workspace, see trioseq_batch_slabs; one of an
+ * affine plan whose records exceed the budget at its planes, see trioseq_plan_affine) waits in
  * arrival order until the running launches leave it room. A request larger than the budget
  * completes with ENOMEM (reported by trioseq_poll).
  * plans[0..nplans) are the scoring schemes a request may name by index (e.g. 0 = DNA,

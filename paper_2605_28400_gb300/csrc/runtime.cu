@@ -385,9 +385,10 @@ trioseq_status build_affine_planes(trioseq_plan_s* plan, trioseq_batch_s* bt) {
 // 200-residue triplets, so the tail of a chunk costs little. A triplet whose records exceed the
 // plan's budget runs over planes instead (four planes of 64 bytes per (j, k) cell).
 // lean: the layout to build when the device had no room for a larger one: 1 the smallest chunks, 2 planes.
+// cap: bytes the records may take (a server's admission), where the plan's budget is larger.
 constexpr size_t kAffineChunkInts = (size_t)1 << 30;  // 4 GB
 constexpr size_t kAffineKeep = (size_t)16 << 30;      // bytes of records a plan keeps between calls
-trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt, int lean) {
+trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt, int lean, size_t cap) {
   const size_t n = bt->n;
   bt->seq_bytes = bt->seq.size();
   bt->affine_chunks.clear();
@@ -397,11 +398,13 @@ trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt, int lean)
     const TripDesc& d = bt->desc[t];
     return (double)(d.len[0] + 1) * (d.len[1] + 1) * (d.len[2] + 1);
   };
+  const size_t budget = std::min(plan->slab_budget, cap) / 4;  // ints
   std::vector<int32_t> order(n);
   for (size_t t = 0; t < n; t++) order[t] = (int32_t)t;
   std::vector<std::pair<int32_t, int32_t>> units;
   // Packed: sigma'' >= 0, every value of the pair's grid below 2^15 (engine.h), and -infinity
-  // (4 |gamma|, plus at most three sigma'') below the smallest real value 2^14 - 8 |gamma|.
+  // (4 |gamma|, plus at most three sigma'') below the smallest real value 2^14 - 8 |gamma|; and the records of
+  // every pair's grid (of its maximal lengths) within the budget.
   const int32_t go = -plan->gap_open;
   if (n >= 2 && plan->packed16 && plan->sig2_nonneg &&
       12 * (int64_t)go + 3 * plan->max_abs_sig2 < (1 << 14)) {
@@ -415,10 +418,12 @@ trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt, int lean)
     bool fits = true;
     for (size_t u = 0; u < n && fits; u += 2) {
       const int32_t t0 = order[u], t1 = u + 1 < n ? order[u + 1] : order[u];
-      int64_t gsum = 0;
+      size_t g[3];
       for (int q = 0; q < 3; q++)
-        gsum += std::max(bt->desc[t0].len[q], bt->desc[t1].len[q]);
-      fits = (int64_t)plan->max_abs_sig2 * (gsum + 3) < (1 << 14);
+        g[q] = (size_t)std::max(bt->desc[t0].len[q], bt->desc[t1].len[q]);
+      fits = (int64_t)plan->max_abs_sig2 * (int64_t)(g[0] + g[1] + g[2] + 3) < (1 << 14) &&
+             (g[0] + 1) * ((g[1] + kAffineWJ) / kAffineWJ) * ((g[2] + kAffineWK) / kAffineWK) *
+                     (size_t)(kAffineRecJ + kAffineRecK) <= budget;
       units.emplace_back(t0, t1);
     }
     if (!fits) units.clear();
@@ -444,7 +449,6 @@ trioseq_status build_affine(trioseq_plan_s* plan, trioseq_batch_s* bt, int lean)
   const auto records = [&](const TripDesc& d) {  // ints
     return (size_t)d.nJ * d.nK * (size_t)(d.glen[0] + 1) * (size_t)(kAffineRecJ + kAffineRecK);
   };
-  const size_t budget = plan->slab_budget / 4;
   size_t limit = lean ? 0 : std::min(budget, kAffineChunkInts);
   for (const auto& un : units) {
     const size_t rec = records(bt->desc[un.first]);
@@ -609,7 +613,8 @@ Variant typed_tb_tile(const trioseq_plan_s* plan, const trioseq_triplet* trip, s
 // that had no room for the batch's first one (make_batch): int32 tiles, or pairs on their 8x8 tile; affine
 // gaps as build_affine says.
 trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n,
-                           uint32_t mode, trioseq_batch_s* bt, int lean = 0) {
+                           uint32_t mode, trioseq_batch_s* bt, int lean = 0,
+                           size_t cap = SIZE_MAX) {
   if (!trip && n) return TRIOSEQ_EINVAL;
   if (mode > TRIOSEQ_WITH_TRACEBACK) return TRIOSEQ_EINVAL;
   const bool tb = mode == TRIOSEQ_WITH_TRACEBACK;
@@ -774,7 +779,7 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   }
   if (plan->affine) {
     if (tb) return TRIOSEQ_ENOTIMPL;  // the affine model is score-only on the device
-    return build_affine(plan, bt, lean);
+    return build_affine(plan, bt, lean, cap);
   }
   // 2. Units of work: one triplet, or in packed int16x2 mode two triplets of the same column-task
   //    grid class paired in one unit (the high halves run on the grid of their maximal lengths).
@@ -971,10 +976,16 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
   const size_t nprog = bt->tasks.size() + 64;
   cudaStream_t as = ws.alloc_stream;
   ws.order_after_last_use();  // a buffer that grows is freed only after its last use
-  if (!ws.inputs.ensure(bt->inputs_bytes, as) ||
+  // the records and codes, whose size is the layout's choice (make_batch)
+  const auto place = [&](DevBuf& b, size_t bytes) {
+    bt->no_room = !b.ensure(bytes, as);
+    return !bt->no_room;
+  };
+  if (!ws.inputs.ensure(bt->inputs_bytes, as) || !place(ws.faces, bt->face_ints * sizeof(int32_t)) ||
       !ws.progress.ensure(nprog * sizeof(int32_t), as) ||
       !ws.scores.ensure(std::max<size_t>(bt->n, 1) * sizeof(int32_t), as) ||
-      (tb && (!ws.rows.ensure(bt->rows_bytes, as) ||
+      (tb && (!place(ws.codes, bt->code_words * sizeof(uint32_t)) ||
+              !ws.rows.ensure(bt->rows_bytes, as) ||
               !ws.lens.ensure(std::max<size_t>(bt->tb_trips.size(), 1) * sizeof(int32_t), as))) ||
       (bt->nplanes && !ws.planes.ensure(bt->nplanes * bt->plane_ints * sizeof(int32_t), as)) ||
       (bt->slab && tb && !ws.walkstate.ensure(4 * sizeof(int32_t), as)) ||
@@ -984,10 +995,6 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
        !ws.best64.ensure(std::max<size_t>(bt->n, 1) * sizeof(unsigned long long), as)) ||
       (pinned && !ws.staging.ensure(align_up(bt->inputs_bytes, 256) + results_bytes(bt))))
     return TRIOSEQ_ENOMEM;
-  // the records and codes last: their size is the layout's choice (make_batch)
-  bt->no_room = !ws.faces.ensure(bt->face_ints * sizeof(int32_t), as) ||
-                (tb && !ws.codes.ensure(bt->code_words * sizeof(uint32_t), as));
-  if (bt->no_room) return TRIOSEQ_ENOMEM;
   // On a private allocation stream, the buffers are ready before any launch stream uses them.
   if (ws.own_stream && cudaStreamSynchronize(as) != cudaSuccess)
     return cuda_status(cudaGetLastError());
@@ -1023,20 +1030,28 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
 }
 
 // Build a batch and place it in `ws` (or a workspace of its own). Where the device has no room for the records
-// and codes of the default layout, the layouts that need less are tried before the call fails.
+// and codes of the default layout, the layouts that need less are tried before the call fails. cap: the bytes
+// that a server admitted the launch with; a layout beyond it gives way to a smaller one, if there is one.
 trioseq_status make_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n, uint32_t mode,
                           Workspace* ws, cudaStream_t st, bool pinned,
-                          std::unique_ptr<trioseq_batch_s>* out) {
-  size_t refused = SIZE_MAX;  // bytes of the layout that found no room
+                          std::unique_ptr<trioseq_batch_s>* out, size_t cap = SIZE_MAX) {
+  const int last = plan->affine ? 2 : 1;
+  size_t least = SIZE_MAX;  // bytes of the smallest layout so far
+  std::unique_ptr<trioseq_batch_s> bt;  // that layout, not yet tried
   trioseq_status s = TRIOSEQ_ENOMEM;
-  for (int lean = 0; lean <= (plan->affine ? 2 : 1); lean++) {
-    std::unique_ptr<trioseq_batch_s> bt(new (std::nothrow) trioseq_batch_s());
-    if (!bt) return TRIOSEQ_ENOMEM;
-    if (const trioseq_status b = build_batch(plan, trip, n, mode, bt.get(), lean); b != TRIOSEQ_OK)
-      return b;
-    const size_t bytes = 4 * (bt->face_ints + (mode == TRIOSEQ_WITH_TRACEBACK ? bt->code_words : 0) +
-                              bt->nplanes * bt->plane_ints);
-    if (bytes >= refused) continue;
+  for (int lean = 0; lean <= last; lean++) {
+    std::unique_ptr<trioseq_batch_s> next(new (std::nothrow) trioseq_batch_s());
+    if (!next) return TRIOSEQ_ENOMEM;
+    s = build_batch(plan, trip, n, mode, next.get(), lean, cap);
+    if (s != TRIOSEQ_OK) return s;
+    const size_t bytes = 4 * (next->face_ints + next->nplanes * next->plane_ints +
+                              (mode == TRIOSEQ_WITH_TRACEBACK ? next->code_words : 0));
+    if (bytes < least) {
+      least = bytes;
+      bt = std::move(next);
+    }
+    s = TRIOSEQ_ENOMEM;
+    if (!bt || (least > cap && lean < last)) continue;
     if (!ws) {
       bt->own_ws.reset(new (std::nothrow) Workspace());
       if (!bt->own_ws) return TRIOSEQ_ENOMEM;
@@ -1044,9 +1059,12 @@ trioseq_status make_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, siz
     }
     bt->ws = ws ? ws : bt->own_ws.get();
     s = upload(bt.get(), st, pinned);
-    if (s == TRIOSEQ_OK) *out = std::move(bt);
-    if (s == TRIOSEQ_OK || !bt->no_room) return s;
-    refused = bytes;
+    if (s == TRIOSEQ_OK) {
+      *out = std::move(bt);
+      return s;
+    }
+    if (!bt->no_room) return s;
+    bt.reset();
     if (ws) {  // what the larger layout did get
       ws->faces.reset();
       ws->codes.reset();
@@ -1911,35 +1929,76 @@ struct SrvSlot {
   trioseq_status launch_st = TRIOSEQ_OK;
 };
 
-// Device bytes one request adds to a launch's workspace (boundary records, flags, and in
-// traceback mode the code stream and rows).
-size_t request_bytes(const trioseq_plan_s* plan, uint32_t mode, const uint32_t len[3]) {
-  const bool tb = mode == TRIOSEQ_WITH_TRACEBACK;
-  Variant v = tb ? plan->tb_variant : plan->score_variant;
-  if (auto_tile(plan, tb) && tb && plan->atype != kGlobal) v = Variant{4, 4};  // typed_tb_tile's larger one
-  const size_t WJ = (size_t)kPR * v.nj, WK = (size_t)kPC * v.nk, W = (size_t)v.nj * v.nk / 8;
+// Device bytes one request adds to a launch's workspace (boundary records, flags, inputs, and in traceback
+// mode the code stream and rows): the most of the tiles that its launch may run on. kLean: the plan's own tile
+// alone, to which make_batch falls back. kGroup: a launch with others, whose tasks together decide the tile, or
+// which pairs it with one of them. Half of a pair on this request's own lengths is counted: one on the maximal
+// lengths of unlike requests, or on the 4x4 tile of a launch of few tasks, may take more, and make_batch then
+// keeps to what was admitted.
+enum class Launch { kLean, kAlone, kGroup };
+size_t request_bytes(const trioseq_plan_s* plan, uint32_t mode, const uint32_t len[3], Launch in) {
+  const bool tb = mode == TRIOSEQ_WITH_TRACEBACK, group = in == Launch::kGroup;
+  const bool own = in != Launch::kLean && auto_tile(plan, tb);
   const size_t a = len[0], b = len[1], c = len[2];
-  const size_t nJ = (b + 1 + WJ - 1) / WJ, nK = (c + 1 + WK - 1) / WK, T = a + 1 + 10;
-  size_t bytes = 4 * nJ * nK * (a + 1) * ((WK + 4) + WJ) + 4 * nJ * nK + 256 + a + b + c + 48;
-  if (tb) bytes += 4 * nJ * nK * T * 32 * W;
-  if (auto_tile(plan, tb) && vl_admits(plan, tb)) {  // the two-per-register tile it may run on instead
-    const size_t t16 = (b + 16) / 16 * ((c + 64) / 64), t32 = (b + 32) / 32 * ((c + 64) / 64);
-    const bool narrow = t16 <= 2 * (size_t)plan->sms;
-    const size_t vt = narrow ? t16 : t32, cells = narrow ? 16 * 64 : 32 * 64;
-    const size_t need = vt * (a + 19) * (4 * (vl_rec_j(4) + kVlRecK) + (tb ? cells / 2 : 0)) +
-                        4 * vt + 256 + a + b + c + 48;
-    bytes = std::max(bytes, need);
+  const auto tasks = [&](const Variant& v) {
+    const size_t WJ = (size_t)kPR * v.nj, WK = (size_t)kPC * v.nk;
+    return ((b + WJ) / WJ) * ((c + WK) / WK);
+  };
+  // records of `slices` slices or steps of `ints` int32, codes of `steps` steps, flag and queue entry
+  const auto sum = [&](const Variant& v, size_t slices, size_t ints, size_t steps) {
+    const size_t cells = (size_t)kPR * v.nj * kPC * v.nk;
+    return tasks(v) * (4 * slices * ints + (tb ? steps * cells / 2 : 0) + 4 + sizeof(Task));
+  };
+  const auto by_slice = [&](const Variant& v) {  // int32 records
+    return sum(v, a + 1, kPC * v.nk + 4 + kPR * v.nj, a + 11);
+  };
+  const auto by_step = [&](const Variant& v) {  // two cells per register
+    return sum(v, a + 19, vl_rec_j(v.nk / 2) + kVlRecK, a + 19);
+  };
+  const auto half_pair = [&](const Variant& v) {  // two triplets per register
+    return sum(v, a + 11, vp_rec_j(v.nk) + vp_rec_k(v.nj), 0) / 2;
+  };
+  const Variant v = tb ? plan->tb_variant : plan->score_variant;
+  size_t bytes = by_slice(v);
+  if (v.vl && in != Launch::kLean) bytes = std::max(bytes, by_step(v));
+  if (own && tb && plan->atype != kGlobal) bytes = std::max(bytes, by_slice(Variant{4, 4}));
+  if (own && vl_admits(plan, tb)) {
+    const bool narrow = tasks(Variant{4, 8, 1}) <= 2 * (size_t)plan->sms;
+    if (narrow) bytes = std::max(bytes, by_step(Variant{4, 8, 1}));
+    if (!narrow || group) bytes = std::max(bytes, by_step(Variant{8, 8, 1}));
   }
-  if (tb) bytes += 3 * (a + b + c) + 64;
-  return bytes;
+  if (own && group && !tb && plan->atype == kGlobal && plan->sig2_nonneg)
+    bytes = std::max(bytes, half_pair(Variant{8, 4}));
+  return bytes + a + b + c + 48 + sizeof(TripDesc) + 256 + (tb ? 3 * (a + b + c) + 64 : 0);
 }
 
-// The same request launched alone: a global-type triplet whose one-launch workspace exceeds the
-// plan's slab budget runs in slabs within that budget (build_batch), so it needs no more.
-size_t request_bytes_alone(const trioseq_plan_s* plan, uint32_t mode, const uint32_t len[3]) {
-  const size_t full = request_bytes(plan, mode, len);
-  return plan->atype == kGlobal ? std::min(full, std::max<size_t>(plan->slab_budget, 1 << 20))
-                                : full;
+// Estimates of one request on a server of `budget` bytes, for a launch with others and for one alone.
+//  * A global-type triplet whose one-launch workspace exceeds the plan's slab budget runs in slabs within that
+//    budget when alone (build_batch), so it needs no more.
+//  * One that fits the server's budget on the plan's own tile is not refused for the larger records of
+//    another: make_batch keeps the launch to what was admitted where it can.
+//  * Affine gaps: the records, or the planes where a triplet's records exceed the budget; over planes every
+//    triplet of a launch would take as much as the largest, so such a request joins no other.
+void estimate(const trioseq_plan_s* plan, const uint32_t len[3], size_t budget, SrvReq* r) {
+  size_t lean = request_bytes(plan, r->mode, len, Launch::kLean);
+  if (plan->affine) {
+    const size_t a = len[0], b = len[1], c = len[2];
+    const size_t tasks = ((b + kAffineWJ) / kAffineWJ) * ((c + kAffineWK) / kAffineWK);
+    const size_t rest = a + b + c + 48 + sizeof(TripDesc) + 512 + tasks * (4 + sizeof(Task));
+    const size_t rec = 4 * tasks * (a + 1) * (size_t)(kAffineRecJ + kAffineRecK) + rest;
+    const bool fits = rec <= std::min(plan->slab_budget, budget);
+    r->bytes = fits ? rec : SIZE_MAX / 4;
+    r->bytes_alone = fits ? rec : 256 * (b + 1) * (c + 1) + rest;
+  } else {
+    r->bytes = request_bytes(plan, r->mode, len, Launch::kGroup);
+    r->bytes_alone = request_bytes(plan, r->mode, len, Launch::kAlone);
+    if (plan->atype == kGlobal) {
+      const size_t slabs = std::max<size_t>(plan->slab_budget, 1 << 20);
+      r->bytes_alone = std::min(r->bytes_alone, slabs);
+      lean = std::min(lean, slabs);
+    }
+  }
+  if (lean <= budget) r->bytes_alone = std::min(r->bytes_alone, budget);
 }
 
 size_t workspace_device_bytes(const Workspace& ws) {
@@ -1989,8 +2048,10 @@ trioseq_status srv_launch(trioseq_server_s* S, SrvSlot& sl) {
       trips[i].s[q] = sl.reqs[i].s[q].data();
       trips[i].len[q] = (uint32_t)sl.reqs[i].s[q].size();
     }
+  // (a small launch may take a few MB more than its estimate: less than the device's pool rounds to)
+  const size_t cap = std::max(sl.bytes, std::min<size_t>(S->budget, (size_t)32 << 20));
   trioseq_status st =
-      make_batch(plan, trips.data(), trips.size(), mode, &sl.ws, sl.stream, true, &sl.batch);
+      make_batch(plan, trips.data(), trips.size(), mode, &sl.ws, sl.stream, true, &sl.batch, cap);
   if (st != TRIOSEQ_OK) return st;
   trioseq_batch_s* bt = sl.batch.get();
   NvtxRange range("trioseq_server_launch");
@@ -2215,8 +2276,7 @@ trioseq_status trioseq_submit(trioseq_server_t S, const trioseq_triplet* t, int3
     if ((int64_t)std::max(plan->max_abs_sig2, plan->atype != kGlobal ? -2 * plan->gap : 0) *
             sumlen >= (1LL << 26) - 1)
       return TRIOSEQ_EOVERFLOW;
-    r.bytes = request_bytes(plan, mode, t->len);
-    r.bytes_alone = request_bytes_alone(plan, mode, t->len);
+    estimate(plan, t->len, S->budget, &r);
     {
       std::lock_guard<std::mutex> lk(S->mu);
       if (S->stop) return TRIOSEQ_EINVAL;
