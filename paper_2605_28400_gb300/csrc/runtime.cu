@@ -50,14 +50,21 @@ struct NvtxRange {
 };
 
 // Host-side fault injection for tests: with TRIOSEQ_TEST_FAIL_ALLOC=N at trioseq_plan, the N-th
-// device allocation after it fails as if the device were out of memory.
-std::atomic<long> g_alloc_calls{0};
-std::atomic<long> g_alloc_fail_at{0};
-
-bool injected_alloc_failure() {
-  const long at = g_alloc_fail_at.load(std::memory_order_relaxed);
-  return at > 0 && g_alloc_calls.fetch_add(1, std::memory_order_relaxed) + 1 == at;
-}
+// device allocation after it fails as if the device were out of memory; with TRIOSEQ_TEST_FAIL_PINNED=N the
+// N-th pinned host allocation.
+struct AllocFault {
+  std::atomic<long> calls{0}, fail_at{0};
+  void arm(const char* env) {
+    const char* v = std::getenv(env);
+    calls.store(0);
+    fail_at.store(v ? std::max(0, std::atoi(v)) : 0);
+  }
+  bool hit() {
+    const long at = fail_at.load(std::memory_order_relaxed);
+    return at > 0 && calls.fetch_add(1, std::memory_order_relaxed) + 1 == at;
+  }
+};
+AllocFault g_device_fault, g_pinned_fault;
 
 struct DevBuf {
   void* p = nullptr;
@@ -84,7 +91,7 @@ struct DevBuf {
   bool ensure(size_t bytes, cudaStream_t st = nullptr) {
     if (bytes <= cap && p) return true;
     const size_t want = std::max<size_t>(bytes, 256);
-    if (injected_alloc_failure()) return false;
+    if (g_device_fault.hit()) return false;
     reset();
     const cudaError_t e = st ? cudaMallocAsync(&p, want, st) : cudaMalloc(&p, want);
     if (e != cudaSuccess) {
@@ -114,8 +121,9 @@ struct HostPinned {
     p = nullptr;
     cap = 0;
     const size_t want = std::max<size_t>(bytes, 4096);
-    if (cudaMallocHost(&p, want) != cudaSuccess) {
+    if (g_pinned_fault.hit() || cudaMallocHost(&p, want) != cudaSuccess) {
       cudaGetLastError();
+      p = nullptr;
       return false;
     }
     cap = want;
@@ -136,7 +144,7 @@ struct Workspace {
   DevBuf walkstate; // slab mode: (i, j, k, n) of the traceback walk between slabs
   DevBuf best64;    // semi-global / local traceback: (score, first cell) key per triplet
   DevBuf spans;     // traceback: begin and end cell of each alignment (6 int32)
-  HostPinned staging;  // per-call path: inputs up, then room for the results down
+  HostPinned staging;  // per-call path: inputs up, then room for results down (Staging)
   // Buffers are allocated and freed in this stream's order. Plans and device-resident batches
   // own a private stream here (own_stream); a serving slot uses its launch stream.
   cudaStream_t alloc_stream = nullptr;
@@ -967,10 +975,18 @@ size_t results_bytes(const trioseq_batch_s* bt) {
          (ntb ? align_up(bt->rows_bytes, 64) + align_up(ntb * 4, 64) + align_up(ntb * 24, 64) : 0);
 }
 
+// How a batch's inputs (and results) pass the host: kPageable copies the inputs synchronously from pageable
+// memory (one-off batch creation); kPinned stages them through the workspace's pinned buffer and copies
+// asynchronously on the launch stream (a server's slot, which has a pinned buffer of its own for results);
+// kPinnedBoth also leaves room there for the results (trioseq_align_batch).
+enum class Staging { kPageable, kPinned, kPinnedBoth };
+// Results beyond this many bytes go straight to their destinations: the copies themselves then take longer
+// than the waits that staging saves, and the plan would keep that much pinned memory.
+constexpr size_t kStagedResults = (size_t)16 << 20;
+
 // Size the workspace and copy the inputs of `bt` into it (stream-ordered).
-// `pinned`: stage through the workspace's pinned buffer and copy asynchronously on `st` (the
-// per-call path); otherwise copy synchronously from pageable memory (one-off batch creation).
-trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
+trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, Staging how) {
+  const bool pinned = how != Staging::kPageable;
   Workspace& ws = *bt->ws;
   const bool tb = bt->mode == TRIOSEQ_WITH_TRACEBACK;
   const size_t nprog = bt->tasks.size() + 64;
@@ -992,9 +1008,14 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
       (tb && !ws.spans.ensure(std::max<size_t>(bt->tb_trips.size(), 1) * 6 * sizeof(int32_t),
                               as)) ||
       (tb && plan_atype(bt) != kGlobal &&
-       !ws.best64.ensure(std::max<size_t>(bt->n, 1) * sizeof(unsigned long long), as)) ||
-      (pinned && !ws.staging.ensure(align_up(bt->inputs_bytes, 256) + results_bytes(bt))))
+       !ws.best64.ensure(std::max<size_t>(bt->n, 1) * sizeof(unsigned long long), as)))
     return TRIOSEQ_ENOMEM;
+  if (pinned) {  // without room for the results they are fetched directly
+    const size_t res = how == Staging::kPinnedBoth ? results_bytes(bt) : 0;
+    if (!(res && res <= kStagedResults && ws.staging.ensure(align_up(bt->inputs_bytes, 256) + res)) &&
+        !ws.staging.ensure(bt->inputs_bytes))
+      return TRIOSEQ_ENOMEM;
+  }
   // On a private allocation stream, the buffers are ready before any launch stream uses them.
   if (ws.own_stream && cudaStreamSynchronize(as) != cudaSuccess)
     return cuda_status(cudaGetLastError());
@@ -1033,7 +1054,7 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, bool pinned) {
 // and codes of the default layout, the layouts that need less are tried before the call fails. cap: the bytes
 // that a server admitted the launch with; a layout beyond it gives way to a smaller one, if there is one.
 trioseq_status make_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n, uint32_t mode,
-                          Workspace* ws, cudaStream_t st, bool pinned,
+                          Workspace* ws, cudaStream_t st, Staging how,
                           std::unique_ptr<trioseq_batch_s>* out, size_t cap = SIZE_MAX) {
   const int last = plan->affine ? 2 : 1;
   size_t least = SIZE_MAX;  // bytes of the smallest layout so far
@@ -1058,7 +1079,7 @@ trioseq_status make_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, siz
       if (bt->own_ws->make_own_stream() != cudaSuccess) return cuda_status(cudaGetLastError());
     }
     bt->ws = ws ? ws : bt->own_ws.get();
-    s = upload(bt.get(), st, pinned);
+    s = upload(bt.get(), st, how);
     if (s == TRIOSEQ_OK) {
       *out = std::move(bt);
       return s;
@@ -1497,8 +1518,8 @@ trioseq_status trioseq_plan(const trioseq_scoring* sc, uint32_t max_len_hint, ui
     plan->test_wait_unset = env_int("TRIOSEQ_TEST_WAIT_UNSET", 0) != 0;
     plan->test_poison = env_int("TRIOSEQ_TEST_POISON", 0) != 0;
     plan->data_flags = env_int("TRIOSEQ_DATA_FLAGS", -1);
-    g_alloc_calls.store(0);
-    g_alloc_fail_at.store(std::max(0, env_int("TRIOSEQ_TEST_FAIL_ALLOC", 0)));
+    g_device_fault.arm("TRIOSEQ_TEST_FAIL_ALLOC");
+    g_pinned_fault.arm("TRIOSEQ_TEST_FAIL_PINNED");
     {
       size_t fr = 0, tot = 0;
       if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
@@ -1596,7 +1617,7 @@ trioseq_status trioseq_align_batch(trioseq_plan_t plan, const trioseq_triplet* t
     cudaStream_t st = (cudaStream_t)stream;
     std::unique_ptr<trioseq_batch_s> bt;
     plan->last.reset();
-    trioseq_status s = make_batch(plan, triplets, n, mode, &plan->ws, st, true, &bt);
+    trioseq_status s = make_batch(plan, triplets, n, mode, &plan->ws, st, Staging::kPinnedBoth, &bt);
     if (s != TRIOSEQ_OK) return s;
     s = run(bt.get(), st);
     plan->ws.mark_use(st);  // also after a partial enqueue: destroy waits for what did run
@@ -1642,7 +1663,8 @@ trioseq_status trioseq_batch_create(trioseq_plan_t plan, const trioseq_triplet* 
     *out = nullptr;
     DeviceGuard g(plan->device);
     std::unique_ptr<trioseq_batch_s> bt;
-    const trioseq_status s = make_batch(plan, triplets, n, mode, nullptr, nullptr, false, &bt);
+    const trioseq_status s = make_batch(plan, triplets, n, mode, nullptr, nullptr, Staging::kPageable,
+                                        &bt);
     if (s != TRIOSEQ_OK) return s;
     *out = bt.release();
     return TRIOSEQ_OK;
@@ -1827,7 +1849,7 @@ trioseq_status trioseq_plan_autotune(trioseq_plan_t plan, const trioseq_triplet*
             break;
           }
           bt.ws = &ws;
-          if ((s = upload(&bt, nullptr, false)) != TRIOSEQ_OK ||
+          if ((s = upload(&bt, nullptr, Staging::kPageable)) != TRIOSEQ_OK ||
               (s = run(&bt, nullptr)) != TRIOSEQ_OK ||
               (s = fetch(&bt, nullptr, nullptr)) != TRIOSEQ_OK) {
             result = s;
@@ -2051,7 +2073,8 @@ trioseq_status srv_launch(trioseq_server_s* S, SrvSlot& sl) {
   // (a small launch may take a few MB more than its estimate: less than the device's pool rounds to)
   const size_t cap = std::max(sl.bytes, std::min<size_t>(S->budget, (size_t)32 << 20));
   trioseq_status st =
-      make_batch(plan, trips.data(), trips.size(), mode, &sl.ws, sl.stream, true, &sl.batch, cap);
+      make_batch(plan, trips.data(), trips.size(), mode, &sl.ws, sl.stream, Staging::kPinned,
+                 &sl.batch, cap);
   if (st != TRIOSEQ_OK) return st;
   trioseq_batch_s* bt = sl.batch.get();
   NvtxRange range("trioseq_server_launch");
