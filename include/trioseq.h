@@ -260,21 +260,21 @@ trioseq_status trioseq_batch_profile(trioseq_batch_t batch, int32_t enable);
 trioseq_status trioseq_batch_timing(trioseq_batch_t batch, float ms[2]);
 
 /* trioseq_plan_autotune — pick the kernel variant for a class of work by measuring it.
- * Runs the sample batch (host strings, n >= 1, mode as for trioseq_align_batch) once per
- * candidate — every instantiated register tile per lane (8x8, 4x8, 4x4 cells, i.e. column blocks
- * of 32x64, 16x64 and 16x32 cells per warp, and in traceback mode also 8x4, 32x32 cells; with
- * every sigma'' in [0, 33] also the two-cells-per-register tiles
- * 8x8v, 4x8v and, score only, 8x16, 32x64, 16x64 and 32x128 cells per warp) times, for int32,
- * progress intervals of 4, 8, 16 and 32 steps —
- * times two passes of each with CUDA events on the legacy default stream, and remembers the
- * fastest in the plan for batches of the same mode, the same single-or-batch kind, and the same
- * bit length of the longest sequence. Later batches of that class use it; other classes keep
- * the defaults: where the scheme admits two cells per register, tile 4x8v for batches of at most
- * two 16x64 column tasks per SM and 8x8v beyond; int32 elsewhere (8x8 score-only, 4x8 traceback, 4x4
- * semi-global and local traceback, interval 8), and for some global batches of at most 8 such tasks or of
- * two triplets of which one is a single task; global score batches whose pairs fit 16-bit halves run two
- * triplets per register. Outputs (any may be null) report
- * the choice. The plan's device memory is untouched; a temporary workspace is used.
+ * Runs the sample batch (host strings, n >= 1, mode as for trioseq_align_batch) on what an untuned
+ * plan would take for it and on each candidate that can take it: the register tiles per lane 8x8,
+ * 4x8 and 4x4 (column blocks of 32x64, 16x64 and 16x32 cells per warp) and in traceback mode 8x4
+ * (32x32), int32 or two triplets per register, and with every sigma'' in [0, 33] the
+ * two-cells-per-register tiles 8x8v, 4x8v and, score only, 8x16 (32x128); where progress counts are
+ * published, each at intervals of 4, 8, 16 and 32 steps. Two passes of each are timed with CUDA
+ * events on the legacy default stream. A candidate that beats the untuned choice by more than 2% is
+ * remembered in the plan for batches of the same mode, the same single-or-batch kind, and the same
+ * bit length of the longest sequence; otherwise, and in other classes, batches keep the defaults:
+ * global score batches whose pairs fit 16-bit halves run two triplets per register (tile 8x4; 4x4 for few
+ * or small triplets; 8x8 where their records exceed the plan's budget); else, where the scheme admits two
+ * cells per register, tile 4x8v for batches of at most two 16x64 column tasks per SM and 8x8v beyond; int32
+ * elsewhere (8x8 score-only, 4x8 traceback, 4x4 semi-global and local traceback, interval 8), and for some
+ * global batches of at most 8 such tasks or of two triplets of which one is a single task. Outputs (any may
+ * be null) report the choice. The plan's device memory is untouched; a temporary workspace is used.
  * Errors: EINVAL, EOVERFLOW, ENOMEM, ETIMEOUT, ECUDA. */
 trioseq_status trioseq_plan_autotune(trioseq_plan_t plan, const trioseq_triplet* sample, size_t n,
                                      uint32_t mode, int32_t* tile_j, int32_t* tile_k,

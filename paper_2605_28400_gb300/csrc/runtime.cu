@@ -247,7 +247,8 @@ struct trioseq_plan_s {
     int TI;
   };
   std::map<int, Tuned> tuned;
-  bool tuning = false;     // set while the autotuner forces candidates
+  // Set while the autotuner measures: candidate tiles in `forced`, or (tune_rule) the rules' own choice.
+  bool tuning = false, tune_rule = false;
   Tuned forced{{8, 8}, 8};
 };
 
@@ -636,13 +637,13 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
     uint32_t maxlen = 0;
     for (size_t t = 0; t < n; t++)
       for (int q = 0; q < 3; q++) maxlen = std::max(maxlen, trip[t].len[q]);
-    if (plan->tuning) {
+    if (plan->tuning && !plan->tune_rule) {
       bt->var = plan->forced.var;
       bt->TI = plan->forced.TI;
     } else if (lean) {
       if (!(tb ? plan->tb_forced : plan->score_forced)) bt->var = tb ? Variant{4, 8} : Variant{8, 8};
     } else {
-      auto it = plan->tuned.find(tune_key(mode, n, maxlen));
+      auto it = plan->tune_rule ? plan->tuned.end() : plan->tuned.find(tune_key(mode, n, maxlen));
       if (it != plan->tuned.end()) {
         bt->var = it->second.var;
         bt->TI = it->second.TI;
@@ -681,7 +682,7 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
       ok_vl = rec <= (double)plan->slab_budget && !(tb && n == 1 && plan->slab_slices > 0);
     }
     if (!ok_vl) {
-      if (plan->tuning) return TRIOSEQ_ECUDA;  // the autotuner skips the candidate
+      if (plan->tuning && !plan->tune_rule) return TRIOSEQ_ECUDA;  // the autotuner skips the candidate
       // the int32 defaults
       bt->var = tb ? (plan->atype != kGlobal ? typed_tb_tile(plan, trip, n) : Variant{4, 8}) : Variant{8, 8};
     }
@@ -1812,8 +1813,8 @@ trioseq_status trioseq_plan_autotune(trioseq_plan_t plan, const trioseq_triplet*
       if (ti) *ti = 0;
       return mode == TRIOSEQ_WITH_TRACEBACK ? TRIOSEQ_ENOTIMPL : TRIOSEQ_OK;
     }
-    // candidate tiles per mode; 8x4 exists for traceback keys only
-    // 8x16 and 8x8 with vl: two cells of one triplet per register
+    // What the rules choose by themselves is measured first, so that a tuned plan is not slower than an untuned
+    // one; then the candidate tiles per mode (int32 or pairs, and with vl two cells per register).
     static const Variant kScoreTiles[] = {{8, 8},    {4, 8},     {4, 4},     {8, 16, 1},
                                           {8, 8, 1}, {8, 16, 2}, {8, 16, 3}, {4, 8, 1}};
     static const Variant kTbTiles[] = {{8, 8}, {4, 8}, {4, 4}, {8, 4}, {8, 8, 1}, {4, 8, 1}};
@@ -1829,54 +1830,70 @@ trioseq_status trioseq_plan_autotune(trioseq_plan_t plan, const trioseq_triplet*
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
       return cuda_status(cudaGetLastError());
     trioseq_status result = TRIOSEQ_OK;
-    float best = 3.0e38f;
-    trioseq_plan_s::Tuned bestv{mode == TRIOSEQ_WITH_TRACEBACK ? plan->tb_variant
-                                                               : plan->score_variant,
-                                plan->TI};
+    trioseq_plan_s::Tuned rule{tb_mode ? plan->tb_variant : plan->score_variant, plan->TI}, bestv{};
+    float rule_ms = 3.0e38f, best = 3.0e38f;
+    bool fits = false;  // something could be measured
     {
-      Workspace ws;  // one workspace, grown to the largest candidate
-      plan->tuning = true;
-      for (size_t vi = 0; vi < ntiles; vi++) {
-        const Variant& v = tiles[vi];
+      struct Tuning {  // also on the way out of an exception
+        trioseq_plan_s* plan;
+        explicit Tuning(trioseq_plan_s* p) : plan(p) { plan->tuning = true; }
+        ~Tuning() { plan->tuning = plan->tune_rule = false; }
+      } tuning(plan);
+      Workspace ws;       // one workspace, grown to the largest candidate
+      bool moot = false;  // the last launch publishes no progress: its interval changes nothing
+      // Time of two passes of a candidate, or (null) of the rules' choice, which `rule` then names; skipped
+      // where there is no such kernel for the work, or no room for its records.
+      const auto measure = [&](const trioseq_plan_s::Tuned* v, float* least) -> trioseq_status {
+        plan->tune_rule = v == nullptr;
+        if (v) plan->forced = *v;
+        moot = true;
+        trioseq_batch_s bt;
+        trioseq_status s = build_batch(plan, sample, n, mode, &bt);
+        if (s != TRIOSEQ_OK) return s == TRIOSEQ_ECUDA ? TRIOSEQ_OK : s;
+        bt.ws = &ws;
+        s = upload(&bt, nullptr, Staging::kPageable);
+        if (s != TRIOSEQ_OK) return bt.no_room ? TRIOSEQ_OK : s;
+        moot = bt.packed >= 2 || bt.df;
+        if (!v) rule = trioseq_plan_s::Tuned{bt.var, bt.TI};
+        if ((s = run(&bt, nullptr)) != TRIOSEQ_OK || (s = fetch(&bt, nullptr, nullptr)) != TRIOSEQ_OK)
+          return s;
+        float ms = 0.f;
+        cudaEventRecord(e0, nullptr);
+        for (int rep = 0; rep < 2 && s == TRIOSEQ_OK; rep++) s = run(&bt, nullptr);
+        cudaEventRecord(e1, nullptr);
+        if (s == TRIOSEQ_OK) s = fetch(&bt, nullptr, nullptr);
+        if (s != TRIOSEQ_OK) return s;
+        if (cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) return cuda_status(cudaGetLastError());
+        *least = std::min(*least, ms);
+        fits = true;
+        return TRIOSEQ_OK;
+      };
+      result = measure(nullptr, &rule_ms);
+      for (size_t vi = 0; vi < ntiles && result == TRIOSEQ_OK; vi++) {
         for (int ti : kTI) {
-          if (v.vl && ti != kTI[0]) break;  // it publishes no progress: the interval is moot
-          plan->forced = trioseq_plan_s::Tuned{v, ti};
-          trioseq_batch_s bt;
-          trioseq_status s = build_batch(plan, sample, n, mode, &bt);
-          if (s == TRIOSEQ_ECUDA) continue;  // variant cannot be resident with this alphabet
-          if (s != TRIOSEQ_OK) {
-            result = s;
-            break;
-          }
-          bt.ws = &ws;
-          if ((s = upload(&bt, nullptr, Staging::kPageable)) != TRIOSEQ_OK ||
-              (s = run(&bt, nullptr)) != TRIOSEQ_OK ||
-              (s = fetch(&bt, nullptr, nullptr)) != TRIOSEQ_OK) {
-            result = s;
-            break;
-          }
-          float ms = 0.f;
-          cudaEventRecord(e0, nullptr);
-          for (int rep = 0; rep < 2 && s == TRIOSEQ_OK; rep++) s = run(&bt, nullptr);
-          cudaEventRecord(e1, nullptr);
-          if (s == TRIOSEQ_OK) s = fetch(&bt, nullptr, nullptr);
-          if (s != TRIOSEQ_OK || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
-            result = s != TRIOSEQ_OK ? s : cuda_status(cudaGetLastError());
-            break;
-          }
+          const trioseq_plan_s::Tuned cand{tiles[vi], ti};
+          float ms = 3.0e38f;
+          if ((result = measure(&cand, &ms)) != TRIOSEQ_OK) break;
           if (ms < best) {
             best = ms;
-            bestv = trioseq_plan_s::Tuned{v, ti};
+            bestv = cand;
           }
+          if (moot) break;
         }
-        if (result != TRIOSEQ_OK) break;
       }
-      plan->tuning = false;
+      // once more, as warm as the candidates were
+      if (result == TRIOSEQ_OK) result = measure(nullptr, &rule_ms);
     }
+    if (result == TRIOSEQ_OK && !fits) result = TRIOSEQ_ENOMEM;
+    const bool tuned = best < 0.98f * rule_ms;  // clearly faster than the rules' choice
+    if (!tuned) bestv = rule;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (result != TRIOSEQ_OK) return result;
-    plan->tuned[tune_key(mode, n, maxlen)] = bestv;
+    if (tuned)
+      plan->tuned[tune_key(mode, n, maxlen)] = bestv;
+    else
+      plan->tuned.erase(tune_key(mode, n, maxlen));  // later batches of the class follow the rules
     if (tile_j) *tile_j = bestv.var.nj;
     if (tile_k) *tile_k = bestv.var.nk;
     if (ti) *ti = bestv.TI;
