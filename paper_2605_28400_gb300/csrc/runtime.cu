@@ -229,6 +229,7 @@ struct trioseq_plan_s {
   int TI = 8;
   int64_t wait_ns = 2000000000LL;  // 2 s without progress = give up
   bool test_wait_unset = false;    // test switch: first-wave warps wait on a flag nothing sets
+  bool test_no_records = false;    // test switch: queue task 0 never runs, its records never come
   bool test_poison = false;        // test switch: boundary records start as a large garbage value
   int data_flags = -1;             // TRIOSEQ_DATA_FLAGS: records as readiness flags (-1: chosen)
   bool graphs = true;              // trioseq_batch_run replays a captured CUDA graph
@@ -1198,6 +1199,16 @@ trioseq_status run(trioseq_batch_s* bt, cudaStream_t st) {
       return cuda_status(e);
     p.TI = 1 << 30;
   }
+  if (plan->test_no_records && bt->packed >= 2) {
+    // Test of the bounded waits on records that are their own flags: the launch finds queue task 0 already
+    // taken, with its records filled with the sentinel and released, and nothing ever writes them. Its
+    // consumers give up after wait_ns, theirs on progress words that are then never released.
+    const TripDesc& d0 = bt->desc[bt->tasks[0].trip];
+    if ((e = cudaMemsetAsync(p.faces, 0xff, bt->face_ints * sizeof(int32_t), st)) != cudaSuccess ||
+        (e = cudaMemsetAsync(queue, 1, 1, st)) != cudaSuccess ||
+        (e = cudaMemsetAsync(prog + d0.prog_base, 1, 1, st)) != cudaSuccess)
+      return cuda_status(e);
+  }
   const int warps_per_cta = wavefront_block_threads(bt->packed) / 32;  // resident warps per CTA
   if (plan->test_wait_unset && !bt->slab) {
     // Test of the bounded waits: every first-wave task but queue task 0 waits on a word of the
@@ -1517,6 +1528,7 @@ trioseq_status trioseq_plan(const trioseq_scoring* sc, uint32_t max_len_hint, ui
     plan->pace = env_int("TRIOSEQ_PACE", 1) != 0;
     plan->wait_ns = (int64_t)std::max(1, env_int("TRIOSEQ_WAIT_MS", 2000)) * 1000000LL;
     plan->test_wait_unset = env_int("TRIOSEQ_TEST_WAIT_UNSET", 0) != 0;
+    plan->test_no_records = env_int("TRIOSEQ_TEST_NO_RECORDS", 0) != 0;
     plan->test_poison = env_int("TRIOSEQ_TEST_POISON", 0) != 0;
     plan->data_flags = env_int("TRIOSEQ_DATA_FLAGS", -1);
     g_device_fault.arm("TRIOSEQ_TEST_FAIL_ALLOC");
