@@ -170,8 +170,10 @@ def kernel_source_hash(tile: str) -> str:
     kernel (tile 8x16, or a label ending in 'v', 's' or 't') or the int32 / two-triplets kernel
     family."""
     common = ("wavefront.cuh", "engine.h")
-    own = (("wavefront_vl.cuh", "kernels_vl.cu") if tile.endswith(("v", "s", "t")) or tile == "8x16"
-           else ("kernels.cu", "kernels_packed.cu", "kernels_slab.cu", "kernels_variants.cu"))
+    own = (("wavefront_vl.cuh", "kernels_vl.cu", "kernels_vl_tb.cu", "kernels_vl_types.cu")
+           if tile.endswith(("v", "s", "t")) or tile == "8x16"
+           else ("wavefront_vp.cuh", "kernels.cu", "kernels_packed.cu", "kernels_slab.cu",
+                 "kernels_variants.cu"))
     h = hashlib.sha256()
     for f in common + own:
         with open(os.path.join(ROOT, "paper_2605_28400_gb300", "csrc", f), "rb") as fh:
@@ -209,7 +211,7 @@ def shard_workload(w, world: int, rank: int, B):
 
 def kernel_of(info: dict, n_triplets: int):
     """(tile label, kernel name) of a batch, as the library reports them (trioseq_batch_kernel):
-    e.g. ("8x8v", "wavefront_vl_kernel<8,4,false>") for two column halves of one triplet per
+    e.g. ("8x8v", "wavefront_vl_kernel<8,4,0>") for two column halves of one triplet per
     register, ("8x16s", ...) for its variant with the sigma''(y,z) tile in shared memory."""
     return info["tile_label"], info["kernel"]
 
@@ -812,18 +814,21 @@ def aux_measurements(B, torch, stream, flush, sms, clock_mhz, skip: str, cpu_leg
     plan = B.trioseq_plan(w.scoring.alphabet, w.scoring.sub, w.scoring.gap)
     tuned_tb = B.trioseq_plan_autotune(plan, strs, B.WITH_TRACEBACK)
     bt = B.trioseq_batch_create(plan, strs, B.WITH_TRACEBACK)
+    packing = B.trioseq_batch_info(bt)["packing"]
     sm, km, wk, sc_tb = time_batch(B, torch, bt, 3, 2, stream, flush, len(strs))
     B.trioseq_batch_destroy(bt)
     B.trioseq_plan_destroy(plan)
     kt = statistics.mean(km)
     ach_t = OPS_PER_CELL * w.cells / (kt / 1e3) / 1e12
-    peak_t = sms * lanes * clock_mhz * 1e6 / 1e12
+    peak_t = packing * sms * lanes * clock_mhz * 1e6 / 1e12
     out["batch4096_traceback"] = {
         "workload": "the 4096-triplet batch with 4-bit traceback codes and one walk per triplet",
         "gcups": w.cells / (statistics.mean(sm) / 1e3) / 1e9, "ms_per_step": statistics.mean(sm),
         "kernel_ms": kt, "walk_ms": statistics.mean(wk), "tuned": tuned_tb,
         "identical_scores_to_score_only": [int(x) for x in sc_tb] == [int(x) for x in sc_batched],
-        "roofline": {"bound": "alu", "achieved": ach_t, "peak": peak_t, "unit": "TOPS (int32)",
+        "packing": packing,
+        "roofline": {"bound": "alu", "achieved": ach_t, "peak": peak_t,
+                     "unit": "TOPS (int32)" if packing == 1 else "TOPS (int16x2 lanes)",
                      "frac": ach_t / peak_t,
                      "code_stream_gbs": CODE_BYTES_PER_CELL * w.cells / kt / 1e6},
         "cells": w.cells}
@@ -833,10 +838,10 @@ def aux_measurements(B, torch, stream, flush, sms, clock_mhz, skip: str, cpu_leg
     return out
 
 
-# Affine gaps (natural gap costs): algorithmic int32 work per cell. Each of the 13 reachable
-# states takes the best of its (move, previous state) candidates: 4 moves with two or three
-# residues x 13 states plus 3 single-residue moves x 13 = 91 candidates, an add and a max each.
-AFFINE_OPS_PER_CELL = 2 * 91
+# Affine gaps (natural gap costs): the operations per cell of the push form (affine.cu): 6 additions of
+# substitution scores, 21 maxima of two, 4 of three and 21 fused add-maxima (2 operations each). The
+# definition's 91 (move, previous state) candidates, an add and a max each, would be 182.
+AFFINE_OPS_PER_CELL = 6 + 21 + 2 * 4 + 2 * 21
 
 
 def affine_measurement(B, torch, stream, flush, sms, clock_mhz, lanes):
@@ -851,6 +856,7 @@ def affine_measurement(B, torch, stream, flush, sms, clock_mhz, lanes):
                                  goldens.AFFINE_GAP_OPEN)
     try:
         bt = B.trioseq_batch_create(plan, strs, B.SCORE_ONLY)
+        packing = B.trioseq_batch_info(bt)["packing"]
         sm, km, _, sc = time_batch(B, torch, bt, 3, 1, stream, flush, len(strs))
         B.trioseq_batch_destroy(bt)
     finally:
@@ -866,12 +872,14 @@ def affine_measurement(B, torch, stream, flush, sms, clock_mhz, lanes):
         pass
     kmean = statistics.mean(km)
     ach = AFFINE_OPS_PER_CELL * w.cells / (kmean / 1e3) / 1e12
-    peak = sms * lanes * clock_mhz * 1e6 / 1e12
+    peak = packing * sms * lanes * clock_mhz * 1e6 / 1e12
     return {"workload": f"{w.name}: affine gaps (natural gap costs, alpha -2, gamma "
                         f"{goldens.AFFINE_GAP_OPEN}), score only",
             "gcups": w.cells / (statistics.mean(sm) / 1e3) / 1e9, "kernel_ms": kmean,
             "cells": w.cells, "equals_oracle_first": checked, "kernel": "affine_kernel",
-            "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TOPS (int32)",
+            "packing": packing,
+            "roofline": {"bound": "alu", "achieved": ach, "peak": peak,
+                         "unit": "TOPS (int32)" if packing == 1 else "TOPS (int16x2 lanes)",
                          "frac": ach / peak, "ops_per_cell": AFFINE_OPS_PER_CELL}}
 
 
@@ -1056,7 +1064,7 @@ def main():
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": ("int32" if packing == 1 else
                       "int16x2 (two cells per 32-bit register, each a 16-bit value relative to "
-                      "a per-task base; exact by the range bound, boundary records int32)"
+                      "a per-task base; exact by the range bound)"
                       if len(strs) == 1 else
                       "int16x2 (two triplets per 32-bit register; exact by the range bound)"),
             "data": "synthetic",

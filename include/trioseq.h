@@ -102,12 +102,13 @@ typedef struct trioseq_plan_s* trioseq_plan_t;
  * TRIOSEQ_LOCAL; every call on the plan (batches, autotuner, server) uses that type.
  * Tuning read from the environment when the plan is created (none changes a result):
  * TRIOSEQ_SCORE_TILE forces the score tile ("8x8", "4x8", "4x4", or the two-cells-per-register
- * "8x16", "8x8v", "4x8v", "8x16s", "8x16t"; work those cannot take runs on the int32 8x8 kernel) and
+ * "8x16", "8x8v", "4x8v", "8x16s", "8x16t"; work those cannot take runs on the int32 tiles) and
  * TRIOSEQ_TB_TILE the traceback tile ("8x8", "4x8", "4x4", "8x4", or two cells per register "8x8v",
  * "4x8v"); TRIOSEQ_TI the progress
  * interval (steps between published progress counts, default 8); TRIOSEQ_DATA_FLAGS=1/0 forces
  * the boundary records to act as their own readiness flags in int32 traceback launches, or not (by
- * default they do for one-triplet traceback batches); TRIOSEQ_PACKED=0 disables two values per
+ * default they do for one-triplet batches, and for every batch of the semi-global and local types);
+ * TRIOSEQ_PACKED=0 disables two values per
  * register unless a tile asks for them; TRIOSEQ_GRAPHS=0 graph replay; TRIOSEQ_PACE=0 first-wave pacing; TRIOSEQ_WAIT_MS the
  * bounded waits' limit (default 2000). TRIOSEQ_CTAS_PER_SM (read per batch) caps the resident
  * CTAs per SM.

@@ -125,7 +125,8 @@ struct WaveParams {
   // First-wave pacing (launches of at least two waves of tasks): queue task n < pace_n starts
   // once task 0 (no producers, never waits) has published n * pace_T / pace_n steps at
   // *pace_flag, spreading the first wave's starts, hence its completions, over one task
-  // duration; 0 disables.
+  // duration; 0 disables. (Launches with two values per register, whose records are their own flags, are not
+  // paced: they read these only in the test of the bounded waits.)
   int32_t pace_n, pace_T;
   const int32_t* pace_flag;
   int32_t one;         // 1, as a launch argument (multiply-adds by it stay on the FMA pipe)

@@ -660,11 +660,9 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
       }
     }
   }
-  // Two cells of one triplet per register (wavefront_vl.cuh), variants 8x16 and 8x8v: score-only
-  // alignment of any type with every sigma'' >= 0, max sigma'' <= 33 (the kernel's range
-  // argument),
-  // and boundary records within the slab budget (it has no slab form). Outside the autotuner's
-  // own candidate runs, work it cannot take runs on the int32 8x8 kernel instead.
+  // Two cells of one triplet per register (wavefront_vl.cuh): schemes, types and modes that vl_admits
+  // names, tiles that are built for them, and boundary records within the slab budget (it has no slab form).
+  // Outside the autotuner's own candidate runs, work it cannot take runs on the int32 tiles instead.
   if (bt->var.vl) {
     // (semi-global and local too: their zero axes and floor add steps of -2*alpha, which must
     // also stay <= 33)

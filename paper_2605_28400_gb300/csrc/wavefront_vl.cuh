@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(VlLaunch<NJ, NH, CS, AT, TB>::warps * 32)
     if (lane == 0) task = atomicAdd(p.queue, 1);
     task = __shfl_sync(kFull, task, 0);
     if (task >= p.ntasks) return;
-    if (task < p.pace_n && task > 0) {  // first-wave pacing, as in wavefront_kernel
+    if (task < p.pace_n && task > 0) {  // in the test of the bounded waits alone (WaveParams)
       const int need = (int)((long long)task * p.pace_T / p.pace_n);
       bool okp = true;
       int seen = 0;
