@@ -1050,9 +1050,15 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, Staging how) {
   return TRIOSEQ_OK;
 }
 
+// Device bytes of a batch's records, codes and slab planes: what its layout decides.
+size_t layout_bytes(const trioseq_batch_s& bt) {
+  return 4 * (bt.face_ints + bt.nplanes * bt.plane_ints +
+              (bt.mode == TRIOSEQ_WITH_TRACEBACK ? bt.code_words : 0));
+}
+
 // Build a batch and place it in `ws` (or a workspace of its own). Where the device has no room for the records
 // and codes of the default layout, the layouts that need less are tried before the call fails. cap: the bytes
-// that a server admitted the launch with; a layout beyond it gives way to a smaller one, if there is one.
+// that a server can give the launch; a layout beyond it gives way to a smaller one, if there is one.
 trioseq_status make_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, size_t n, uint32_t mode,
                           Workspace* ws, cudaStream_t st, Staging how,
                           std::unique_ptr<trioseq_batch_s>* out, size_t cap = SIZE_MAX) {
@@ -1065,8 +1071,7 @@ trioseq_status make_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, siz
     if (!next) return TRIOSEQ_ENOMEM;
     s = build_batch(plan, trip, n, mode, next.get(), lean, cap);
     if (s != TRIOSEQ_OK) return s;
-    const size_t bytes = 4 * (next->face_ints + next->nplanes * next->plane_ints +
-                              (mode == TRIOSEQ_WITH_TRACEBACK ? next->code_words : 0));
+    const size_t bytes = layout_bytes(*next);
     if (bytes < least) {
       least = bytes;
       bt = std::move(next);
@@ -1974,7 +1979,8 @@ struct SrvSlot {
   size_t off_err = 0, off_lens = 0, off_rows = 0;
   std::unique_ptr<trioseq_batch_s> batch;
   std::vector<SrvReq> reqs;
-  size_t bytes = 0;  // workspace estimate admitted for the launch on this slot
+  size_t bytes = 0;  // workspace admitted for the launch on this slot: its estimate, then at least what it took
+  size_t cap = 0;    // the estimate and what the budget had left
   trioseq_status launch_st = TRIOSEQ_OK;
 };
 
@@ -1982,8 +1988,8 @@ struct SrvSlot {
 // mode the code stream and rows): the most of the tiles that its launch may run on. kLean: the plan's own tile
 // alone, to which make_batch falls back. kGroup: a launch with others, whose tasks together decide the tile, or
 // which pairs it with one of them. Half of a pair on this request's own lengths is counted: one on the maximal
-// lengths of unlike requests, or on the 4x4 tile of a launch of few tasks, may take more, and make_batch then
-// keeps to what was admitted.
+// lengths of unlike requests, or on the 4x4 tile of a launch of few tasks, may take more; the server counts what
+// the launch then took, and make_batch keeps that to what the budget has left.
 enum class Launch { kLean, kAlone, kGroup };
 size_t request_bytes(const trioseq_plan_s* plan, uint32_t mode, const uint32_t len[3], Launch in) {
   const bool tb = mode == TRIOSEQ_WITH_TRACEBACK, group = in == Launch::kGroup;
@@ -2025,7 +2031,7 @@ size_t request_bytes(const trioseq_plan_s* plan, uint32_t mode, const uint32_t l
 //  * A global-type triplet whose one-launch workspace exceeds the plan's slab budget runs in slabs within that
 //    budget when alone (build_batch), so it needs no more.
 //  * One that fits the server's budget on the plan's own tile is not refused for the larger records of
-//    another: make_batch keeps the launch to what was admitted where it can.
+//    another: make_batch keeps the launch to what the budget has left where it can.
 //  * Affine gaps: the records, or the planes where a triplet's records exceed the budget; over planes every
 //    triplet of a launch would take as much as the largest, so such a request joins no other.
 void estimate(const trioseq_plan_s* plan, const uint32_t len[3], size_t budget, SrvReq* r) {
@@ -2097,11 +2103,9 @@ trioseq_status srv_launch(trioseq_server_s* S, SrvSlot& sl) {
       trips[i].s[q] = sl.reqs[i].s[q].data();
       trips[i].len[q] = (uint32_t)sl.reqs[i].s[q].size();
     }
-  // (a small launch may take a few MB more than its estimate: less than the device's pool rounds to)
-  const size_t cap = std::max(sl.bytes, std::min<size_t>(S->budget, (size_t)32 << 20));
   trioseq_status st =
       make_batch(plan, trips.data(), trips.size(), mode, &sl.ws, sl.stream, Staging::kPinned,
-                 &sl.batch, cap);
+                 &sl.batch, sl.cap);
   if (st != TRIOSEQ_OK) return st;
   trioseq_batch_s* bt = sl.batch.get();
   NvtxRange range("trioseq_server_launch");
@@ -2249,11 +2253,16 @@ void srv_loop(trioseq_server_s* S) {
       }
       sl.bytes = sl.reqs.size() == 1 ? sl.reqs.front().bytes_alone : full;
       S->in_flight += sl.bytes;
+      sl.cap = sl.bytes + (S->budget > S->in_flight ? S->budget - S->in_flight : 0);
       sl.busy = true;
       acted = true;
       lk.unlock();
       sl.launch_st = no_throw([&] { return srv_launch(S, sl); });  // the thread must not throw
       lk.lock();
+      if (sl.batch && layout_bytes(*sl.batch) > sl.bytes) {  // a pair of unlike requests, for instance
+        S->in_flight += layout_bytes(*sl.batch) - sl.bytes;
+        sl.bytes = layout_bytes(*sl.batch);
+      }
       busy_any = true;
     }
     if (S->stop && S->pending.empty() && !busy_any) break;
