@@ -853,7 +853,7 @@ trioseq_status build_batch(trioseq_plan_s* plan, const trioseq_triplet* trip, si
   // 4. Slab mode: one global-type int32 triplet whose boundary records (and, with traceback,
   //    codes) would exceed the plan's budget at once, or any such triplet when a slab height is
   //    forced. The cube then runs slab by slab, each launch seeded from the plane the slab below
-  //    left (DESIGN: linear-space traceback).
+  //    left (linear-space traceback).
   bt->slab = bt->nslab = 0;
   bt->nplanes = bt->plane_ints = 0;
   bt->slab_desc.clear();
