@@ -293,7 +293,7 @@ struct trioseq_batch_s {
   size_t plane_ints = 0, nplanes = 0, off_slab = 0;
   std::vector<TripDesc> slab_desc;
   bool uploaded = false;
-  bool no_room = false;  // the last upload failed for its boundary records or codes
+  bool no_room = false;  // the upload found no room for the boundary records, the codes or the rest
   // results of the last run (host)
   std::vector<uint8_t> h_rows;
   std::vector<int32_t> h_lens;
@@ -992,15 +992,11 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, Staging how) {
   const size_t nprog = bt->tasks.size() + 64;
   cudaStream_t as = ws.alloc_stream;
   ws.order_after_last_use();  // a buffer that grows is freed only after its last use
-  // the records and codes, whose size is the layout's choice (make_batch)
-  const auto place = [&](DevBuf& b, size_t bytes) {
-    bt->no_room = !b.ensure(bytes, as);
-    return !bt->no_room;
-  };
-  if (!ws.inputs.ensure(bt->inputs_bytes, as) || !place(ws.faces, bt->face_ints * sizeof(int32_t)) ||
+  if (!ws.inputs.ensure(bt->inputs_bytes, as)) return TRIOSEQ_ENOMEM;
+  if (!ws.faces.ensure(bt->face_ints * sizeof(int32_t), as) ||
       !ws.progress.ensure(nprog * sizeof(int32_t), as) ||
       !ws.scores.ensure(std::max<size_t>(bt->n, 1) * sizeof(int32_t), as) ||
-      (tb && (!place(ws.codes, bt->code_words * sizeof(uint32_t)) ||
+      (tb && (!ws.codes.ensure(bt->code_words * sizeof(uint32_t), as) ||
               !ws.rows.ensure(bt->rows_bytes, as) ||
               !ws.lens.ensure(std::max<size_t>(bt->tb_trips.size(), 1) * sizeof(int32_t), as))) ||
       (bt->nplanes && !ws.planes.ensure(bt->nplanes * bt->plane_ints * sizeof(int32_t), as)) ||
@@ -1008,8 +1004,10 @@ trioseq_status upload(trioseq_batch_s* bt, cudaStream_t st, Staging how) {
       (tb && !ws.spans.ensure(std::max<size_t>(bt->tb_trips.size(), 1) * 6 * sizeof(int32_t),
                               as)) ||
       (tb && plan_atype(bt) != kGlobal &&
-       !ws.best64.ensure(std::max<size_t>(bt->n, 1) * sizeof(unsigned long long), as)))
+       !ws.best64.ensure(std::max<size_t>(bt->n, 1) * sizeof(unsigned long long), as))) {
+    bt->no_room = true;  // records and codes, or what comes after them: a smaller layout may fit
     return TRIOSEQ_ENOMEM;
+  }
   if (pinned) {  // without room for the results they are fetched directly
     const size_t res = how == Staging::kPinnedBoth ? results_bytes(bt) : 0;
     if (!(res && res <= kStagedResults && ws.staging.ensure(align_up(bt->inputs_bytes, 256) + res)) &&
@@ -1205,7 +1203,7 @@ trioseq_status run(trioseq_batch_s* bt, cudaStream_t st) {
   if (plan->test_no_records && bt->packed >= 2) {
     // Test of the bounded waits on records that are their own flags: the launch finds queue task 0 already
     // taken, with its records filled with the sentinel and released, and nothing ever writes them. Its
-    // consumers give up after wait_ns, theirs on progress words that are then never released.
+    // consumers give up after wait_ns, theirs on the records of those.
     const TripDesc& d0 = bt->desc[bt->tasks[0].trip];
     if ((e = cudaMemsetAsync(p.faces, 0xff, bt->face_ints * sizeof(int32_t), st)) != cudaSuccess ||
         (e = cudaMemsetAsync(queue, 1, 1, st)) != cudaSuccess ||

@@ -1,5 +1,5 @@
-"""A device without room for a batch's boundary records or codes: layouts that need less answer, with the
-same results, before the call fails. The refused allocation is injected on the host
+"""A device without room for a batch's boundary records or codes, or for what comes after them: layouts that
+need less answer, with the same results, before the call fails. The refused allocation is injected on the host
 (TRIOSEQ_TEST_FAIL_ALLOC); nothing else changes on the device."""
 import os
 
@@ -13,8 +13,8 @@ from paper_2605_28400_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 DNA = synth.dna_scoring()
-# the allocations of a batch in their order: inputs, records, progress, scores, codes
-RECORDS, CODES = 2, 5
+# the allocations of a batch in their order: inputs, records, progress, scores, codes, rows
+RECORDS, CODES, ROWS = 2, 5, 6
 
 
 def _plan(fail, gap_open=None, flags=0, **env):
@@ -69,7 +69,8 @@ def test_affine(shapes, kernel, packing):
 
 @pytest.mark.parametrize("flags,okind,label,fail", [
     (B.GLOBAL, oracle.GLOBAL, "4x8", RECORDS), (B.GLOBAL, oracle.GLOBAL, "4x8", CODES),
-    (B.LOCAL, oracle.LOCAL, "4x8", RECORDS)], ids=["records", "codes", "local"])
+    (B.GLOBAL, oracle.GLOBAL, "4x8", ROWS), (B.LOCAL, oracle.LOCAL, "4x8", RECORDS)],
+    ids=["records", "codes", "rows", "local"])
 def test_rows(flags, okind, label, fail):
     # many more steps than slices (a = 3): the default tiles need more room than int32 4x8 here
     trips = _trips([(3, 40, 63)] * 9 + [(5, 33, 60)])

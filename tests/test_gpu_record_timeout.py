@@ -1,6 +1,6 @@
 """Bounded waits on boundary records that are their own readiness flags, in the kernels with two values per
 register. Under TRIOSEQ_TEST_NO_RECORDS a launch finds its first column task taken and its records released
-but never written: the task's consumers get past their start and give up on the records, theirs on the release
+but never written: the task's consumers get past their start and give up on the records, theirs on the records
 of those. No wait lasts longer than 20 ms, the call reports ETIMEOUT, and the same process then aligns
 exactly."""
 import os
